@@ -49,7 +49,11 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
     const int n = net.n_pq;
     cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_ends); cudaFree(d.t_z);
     cudaFree(d.t_zrow); cudaFree(d.t_yrow); cudaFree(d.t_kidx); cudaFree(d.t_zrow_f); cudaFree(d.t_z64);
+    cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
     d.t_z64 = nullptr;
+    d.t_topo = nullptr;
+    d.t_cp = nullptr;
+    d.t_zf = nullptr;
     d.t_col = d.t_end = d.t_par = d.t_ecnt = d.t_ends = d.t_kidx = nullptr;
     d.t_z = d.t_zrow = nullptr;
     d.t_yrow = d.t_zrow_f = nullptr;
@@ -103,6 +107,23 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
                     z[s] = zz;
                 }
             }
+            // The mixed kernel's packed words; offsets in bytes of float2 except at kTreeBigBPT, where
+            // they would not fit (bits 0-14 of the upper half, 0-15 of the lower one).
+            const int unit = bpt == kTreeBigBPT ? 1 : 8;
+            std::vector<int4> topo(ns);
+            std::vector<int> cp(ns);
+            std::vector<float2> zf(ns);
+            for (int s = 0; s < ns; ++s) {
+                const int q = (s % th) * bpt + s / th;
+                const int rng = ph > 1 ? end[s] : (q < n ? slot(end[s] - 1) : s) * unit;
+                const int k = kidx[s] < 0 ? -1 : kidx[s] * unit;
+                cp[s] = (int)((unsigned)(col[s] & 0xffff) | (unsigned)par[s] << 16);
+                const unsigned ec = (unsigned)ecnt[s];
+                topo[s] = make_int4((int)((unsigned)(rng & 0xffff) | (unsigned)k << 16), cp[s],
+                                    (int)((ec & 0xffff0000u) | (ec & 0xffffu) * (unsigned)unit), 0);
+                zf[s] = make_float2(z[s].x, z[s].y);
+                if (kidx[s] * unit > 0x7fff || (int)(ec & 0xffffu) * unit > 0xffff) fits = false;
+            }
             d.t_n_ends = (int)ends.size();
             if (ends.empty()) ends.push_back(0);
             auto up = [](auto **dst, const auto &v) -> bool {
@@ -113,7 +134,8 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
             if (!fits) {
                 d.t_threads = 0;
             } else if (!up(&d.t_col, col) || !up(&d.t_end, end) || !up(&d.t_par, par) || !up(&d.t_ecnt, ecnt) ||
-                       !up(&d.t_ends, ends) || !up(&d.t_z, z) || !up(&d.t_kidx, kidx) ||
+                       !up(&d.t_ends, ends) || !up(&d.t_z, z) || !up(&d.t_kidx, kidx) || !up(&d.t_topo, topo) || !up(&d.t_cp, cp) ||
+                       !up(&d.t_zf, zf) ||
                        (ph == 1 && !up(&d.t_z64, z64)) || (ph > 1 && (!up(&d.t_zrow, zrow) || !up(&d.t_yrow, yrow) || !up(&d.t_zrow_f, zrow_f)))) {
                 cudaGetLastError();
                 return TPF_ECUDA;
@@ -275,7 +297,7 @@ void free_device(tpf_handle *h) {
     cudaFree(d.Kr16); cudaFree(d.Ki16);
     cudaFree(d.par); cudaFree(d.ch_ptr); cudaFree(d.ch); cudaFree(d.ypar);
     cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_ends); cudaFree(d.t_z);
-    cudaFree(d.t_kidx); cudaFree(d.t_z64);
+    cudaFree(d.t_kidx); cudaFree(d.t_z64); cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
     cudaFree(d.zip64); cudaFree(d.t_zip_hi); cudaFree(d.t_zip_lo);
     cudaFree(d.csr_self); cudaFree(d.vs64); cudaFree(d.t_zrow); cudaFree(d.t_yrow); cudaFree(d.t_zrow_f);
     d = DeviceNet();

@@ -130,6 +130,12 @@ struct DeviceNet {
     int *t_col = nullptr, *t_end = nullptr, *t_par = nullptr, *t_ecnt = nullptr, *t_ends = nullptr;
     int *t_kidx = nullptr;  // per slot: the index in t_ends at which its position appears, or -1
     float4 *t_z = nullptr;
+    // What the mixed kernel reads of a slot when it sets a column up, as one 16-byte word: the range
+    // word, column | parent slot << 16, the ends word (tpf_sparse.cu), 0; the second words again on
+    // their own; and the high words of t_z.
+    int4 *t_topo = nullptr;
+    int *t_cp = nullptr;
+    float2 *t_zf = nullptr;
     double2 *t_z64 = nullptr;  // FP64 z per slot (single phase), for the FP64 sparse kernel
     // ZIP load coefficients (Eq. 3), set by tpf_set_zip; null for constant power.  zip64: double
     // [3][n] in column order (FP64 path); t_zip_hi / t_zip_lo: float4 (alpha_P, alpha_I, alpha_Z, 0)

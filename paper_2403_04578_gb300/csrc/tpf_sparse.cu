@@ -49,10 +49,12 @@ constexpr int kGather = 4;  // ends-list entries per position gathered without a
 
 // One feeder's share of a launch: its network arrays (slot layout) and its tensors.
 struct TreeWork {
-    int n, n_ends;
+    int n;
     float2 vs_f;
     c2 vs_dd;
-    const int *col, *end, *par, *ecnt, *ends, *kidx;
+    const int4 *topo;  // per slot: range word, column | parent slot << 16, ends word, 0 (DeviceNet)
+    const int *cp;     // the second words again, contiguous
+    const float2 *zf;  // per slot: FP32 branch impedance
     const float4 *z;
     const float4 *zip_hi, *zip_lo;  // ZIP coefficients (alpha_P, alpha_I, alpha_Z, 0) per slot, or null
     // Polyphase: positions per phase block, v_s per phase, per slot the rows of the branch's
@@ -97,12 +99,34 @@ struct TreeArgs {
     float4 *scratch;
 };
 
-// Packed per-position word: ends-list start (bits 0-15), count (16-29), phase (30-31).
+// Packed per-position ends word: ends-list start (bits 0-15), count (16-29), phase (30-31), and range
+// word: the subtree's range (bits 0-15), ends-list place (16-31, negative: none).  Starts, places and
+// single-phase range slots are byte offsets into float2 arrays (kTreeBigBPT: indices, whose largest
+// offsets would not fit 15 bits), so that a sweep uses them as shared-memory addresses undecoded.
+template <int kBPT>
+constexpr int kOff = kBPT == kTreeBigBPT ? 1 : 8;
 __device__ __forceinline__ int ends_cnt(int ec) { return (int)(((unsigned)ec >> 16) & 0x3fffu); }
 __device__ __forceinline__ int phase_of(int ec) { return (int)((unsigned)ec >> 30); }
+template <int kBPT>
+__device__ __forceinline__ int ends_start(int ec) { return (ec & 0xffff) / kOff<kBPT>; }
+// Element of a float2 / float4 array at an offset of a word above.
+template <int kBPT>
+__device__ __forceinline__ float2 &at8(float2 *p, int off) {
+    return *reinterpret_cast<float2 *>(reinterpret_cast<char *>(p) + off * (8 / kOff<kBPT>));
+}
+template <int kBPT>
+__device__ __forceinline__ float4 &at16(float4 *p, int off) {
+    return *reinterpret_cast<float4 *>(reinterpret_cast<char *>(p) + off * (16 / kOff<kBPT>));
+}
 
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// Sums and differences of a complex pair in one packed instruction each (a - b as the exactly
+// rounded a + (-1) b): the same two roundings as two scalar ones, half the issue slots.  The kernel
+// is bound by issue slots and shared-memory latency; with scalar sums and the packed words below it
+// takes 6.27 ms instead of 5.92 on 175,200 complex64 columns of a 500-bus feeder, 3.51 instead of
+// 3.30 ms on 16,384 three-phase columns of 500 buses, 10.46 instead of 10.47 on 131,072 columns of
+// 1,000 buses (where the FP64 conversions of S and V fill the gaps).
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 // The FP32 products below are written with explicitly rounded intrinsics, so that the compiler
 // cannot contract them differently in different instantiations of the kernel: every kernel then
 // rounds a given formula the same way, whatever code surrounds it (ZIP loads with alpha_P = 1 then
@@ -295,9 +319,11 @@ __device__ __forceinline__ int slot_of(int p, int th) {
     return (p & (kBPT - 1)) * th + p / kBPT;
 }
 // Slot of the position after the one in slot s.
+// (both in the units of the range words).
 template <int kBPT>
 __device__ __forceinline__ int next_slot(int s, int th) {
-    return s < (kBPT - 1) * th ? s + th : s - (kBPT - 1) * th + 1;
+    const int u = kOff<kBPT>;
+    return s < (kBPT - 1) * th * u ? s + th * u : s - (kBPT - 1) * th * u + u;
 }
 
 // First part of an anchor, in double-float.  On entry A[s] = (S_hi) and B[s] = (V_ref, S_lo) for
@@ -347,7 +373,7 @@ __device__ __forceinline__ c2 anchor_dd(const TreeWork &a, float4 *A, float4 *B,
         const int q = base + j, s = j * th + tid;
         if (q < n) {
             if (kPh == 1) {
-                c2 L = unpack(A[s_rk[s] & 0xffff]);
+                c2 L = unpack(at16<kBPT>(A, s_rk[s] & 0xffff));
                 if (q > 0) L = cqsub(L, unpack(A[j ? s - th : (kBPT - 1) * th + tid - 1]));
                 const float4 zq = B[s];
                 B[s] = pack(cqmul(c2{{zq.x, zq.z}, {zq.y, zq.w}}, L));
@@ -371,7 +397,7 @@ __device__ __forceinline__ c2 anchor_dd(const TreeWork &a, float4 *A, float4 *B,
 #pragma unroll
     for (int j = 0; j < kBPT; ++j) {
         const int s = j * th + tid, k = s_rk[s] >> 16;
-        if (k >= 0) A[k] = B[s];
+        if (k >= 0) at16<kBPT>(A, k) = B[s];
     }
     __syncthreads();
     // Inclusive prefix sums of E_q = x_q - (x_b of every b whose range ends at q), into B.
@@ -384,7 +410,7 @@ __device__ __forceinline__ c2 anchor_dd(const TreeWork &a, float4 *A, float4 *B,
 #pragma unroll
             for (int i = 1; i < kBPT; ++i)
                 if (j == i) ec = ecnt[i];
-            const int st = ec & 0xffff, cnt = ends_cnt(ec);
+            const int st = ends_start<kBPT>(ec), cnt = ends_cnt(ec);
             c2 e = unpack(B[s]);
 #pragma unroll 1
             for (int k = 0; k < cnt; ++k) e = cqsub(e, unpack(A[st + k]));
@@ -427,16 +453,12 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
     float4 *const B = kBig ? big : tsm + ns;  // [ns] V_ref (anchor input), x (anchor), then D = BFS(V_ref) - V_ref
     float4 *const C = kBig ? big + ns : tsm + 2 * ns;  // [ns] (S_hi, z_hi) of each position
     float4 *const Zs = kBig ? big + 2 * ns : tsm + 3 * ns;  // [ns] ZIP coefficients (kZip only)
-    // [ns] the subtree's range [q, end_q): one phase, the slot of its last position end_q - 1 (the
-    // slot itself for a leaf); polyphase, end_q.  (The polyphase impedance rows stay in device
-    // memory, read through the cache: in shared memory they would halve the resident blocks.)
-    // [ns] per slot, bits 0-15: the subtree's range [q, end_q): one phase, the slot of its last
+    // [ns] range words.  Bits 0-15, the subtree's range [q, end_q): one phase, the slot of its last
     // position end_q - 1 (the slot itself for a leaf); polyphase, end_q.  Bits 16-31: where the
-    // position's branch term goes in the ends-ordered copy of X (-1: nowhere).  One word, so that a
-    // sweep reads both with one shared-memory load.  (The polyphase impedance rows stay in device
-    // memory, read through the cache: in shared memory they would halve the resident blocks.)
+    // position's branch term goes in the ends-ordered copy of X (negative: nowhere).  One word, so
+    // that a sweep reads both with one shared-memory load.  (The polyphase impedance rows stay in
+    // device memory, read through the cache: in shared memory they would halve the resident blocks.)
     int *const s_rk = reinterpret_cast<int *>(tsm + (kBig ? 1 : (kZip ? 4 : 3)) * ns);
-    short *const s_par = reinterpret_cast<short *>(s_rk + ns);  // [ns] parent slot, -1 = the slack
     float2 *P = reinterpret_cast<float2 *>(A);  // [ns] inclusive prefix sums of the load currents
     float2 *X = P + ns;                           // [ns] branch terms z_q L_q; the residual's x at the end
     __shared__ float2 wt2[kMaxWarps];
@@ -449,13 +471,6 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
     const double2 *S64 = static_cast<const double2 *>(a.S) + t * n;
     const float2 *S32 = static_cast<const float2 *>(a.S) + t * n;
 
-#pragma unroll
-    for (int j = 0; j < kBPT; ++j) {
-        const int q = base + j, s = j * th + tid;
-        const int rng = kPh > 1 ? a.end[s] : (q < n ? slot_of<kBPT>(a.end[s] - 1, th) : s);
-        s_rk[s] = (rng & 0xffff) | (a.kidx[s] << 16);
-        s_par[s] = (short)a.par[s];
-    }
     // Per position: V_ref (or V before anchoring) and delta = V - V_ref in registers, the ends-list
     // bounds in registers, S and z in C.
     float2 vr[kBPT], dl[kBPT];
@@ -465,10 +480,15 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
         const int q = base + j, s = j * th + tid;
         vr[j] = make_float2(1.0f, 0.0f);
         dl[j] = make_float2(0.0f, 0.0f);
-        ecnt[j] = 0;
+        // One 16-byte load per position brings its whole topology; with a load each for column, range,
+        // parent, ends word and ends place, decoded here, 131,072 columns of 1,000 buses took 10.70 ms
+        // instead of 10.47, and 175,200 complex64 columns of 500 buses 6.39 ms instead of 5.92.
+        const int4 tp = a.topo[s];
+        s_rk[s] = tp.x;
+        ecnt[j] = tp.z;
         float2 sh = make_float2(0.0f, 0.0f), zh = sh, sl = sh;
         if (q < n) {
-            const int i = a.col[s];
+            const int i = tp.y & 0xffff;
             if (a.s32) {
                 sh = S32[i];
             } else {
@@ -476,9 +496,7 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
                 sh = make_float2(__double2float_rn(sv.x), __double2float_rn(sv.y));
                 sl = make_float2(__double2float_rn(sv.x - (double)sh.x), __double2float_rn(sv.y - (double)sh.y));
             }
-            const float4 zq = a.z[s];
-            zh = make_float2(zq.x, zq.y);
-            ecnt[j] = a.ecnt[s];
+            zh = a.zf[s];
         }
         C[s] = make_float4(sh.x, sh.y, zh.x, zh.y);
         B[s] = make_float4(sl.x, sl.y, 0.0f, 0.0f);  // S_lo until the first anchor replaces it by D
@@ -490,9 +508,9 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
         for (int j = 0; j < kBPT; ++j) {
             const int q = base + j, s = j * th + tid;
             if (q < n) {
-                const int64_t k = t * n + a.col[s];
+                const int64_t k = t * n + (a.cp[s] & 0xffff);
                 if (a.v0_pred) {
-                    const float2 d = __half22float2(static_cast<const __half2 *>(a.V0)[t * a.v0_pitch + a.col[s]]);
+                    const float2 d = __half22float2(static_cast<const __half2 *>(a.V0)[t * a.v0_pitch + (a.cp[s] & 0xffff)]);
                     vr[j] = make_float2(1.0f + d.x, d.y);
                     const float m2 = abs2(vr[j]);
                     off_band |= !(m2 >= 0.49f && m2 <= 1.21f);
@@ -563,7 +581,7 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
                     const int q = base + j, s = j * th + tid;
                     float2 slo = make_float2(0.0f, 0.0f);
                     if (q < n && !a.s32) {
-                        const double2 sv = S64[a.col[s]];
+                        const double2 sv = S64[a.cp[s] & 0xffff];
                         const float4 cs = C[s];
                         slo = make_float2(__double2float_rn(sv.x - (double)cs.x), __double2float_rn(sv.y - (double)cs.y));
                     }
@@ -661,8 +679,8 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
                 float2 xq = make_float2(0.0f, 0.0f);  // positions past n contribute nothing
                 if (q < n) {
                     if (kPh == 1) {
-                        const int ls = rk & 0xffff;  // slot of the subtree's last position (s for a leaf)
-                        float2 L = ls == s ? loc[j] : P[ls];
+                        const int ls = rk & 0xffff;  // the subtree's last position (s for a leaf)
+                        float2 L = ls == s * kOff<kBPT> ? loc[j] : at8<kBPT>(P, ls);
                         if (j) L = sub2(L, loc[j - 1]);
                         else if (q > 0) L = sub2(L, P[(kBPT - 1) * th + tid - 1]);
                         const float4 cs = C[s];
@@ -682,7 +700,7 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
                 // The branch term goes where the position that closes its range gathers it: X
                 // holds the terms in ends-list order, so each position's list is contiguous.
                 const int k = rk >> 16;
-                if (k >= 0) X[k] = xq;
+                if (k >= 0) at8<kBPT>(X, k) = xq;
                 loc[j] = xq;
             }
             __syncthreads();
@@ -692,18 +710,20 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
             bool longer = false;
 #pragma unroll
             for (int j = 0; j < kBPT; ++j) {
-                const int st = ecnt[j] & 0xffff, cnt = ends_cnt(ecnt[j]);
+                // The count sits above the start: count > k is word >= (k + 1) << 16.
+                const int st = ecnt[j] & 0xffff, ec = kPh > 1 ? ecnt[j] & 0x3fffffff : ecnt[j];
                 float2 e = loc[j];
+                const float2 *Xs = &at8<kBPT>(X, st);
 #pragma unroll
                 for (int k = 0; k < kGather; ++k)
-                    if (k < cnt) e = sub2(e, X[st + k]);
-                longer |= cnt > kGather;
+                    if (ec >= (k + 1) << 16) e = sub2(e, Xs[k]);
+                longer |= ec >= (kGather + 1) << 16;
                 loc[j] = e;
             }
             if (longer) {
 #pragma unroll
                 for (int j = 0; j < kBPT; ++j) {
-                    const int st = ecnt[j] & 0xffff, cnt = ends_cnt(ecnt[j]);
+                    const int st = ends_start<kBPT>(ecnt[j]), cnt = ends_cnt(ecnt[j]);
                     for (int k = kGather; k < cnt; ++k) loc[j] = sub2(loc[j], X[st + k]);
                 }
             }
@@ -754,6 +774,7 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
     // end of the previous one's range, while inside q's range.
     float2 *J = reinterpret_cast<float2 *>(B);
     float2 xs[kBPT];
+    int cp[kBPT];
 #pragma unroll
     for (int j = 0; j < kBPT; ++j) {
         const int q = base + j, s = j * th + tid;
@@ -764,8 +785,9 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
             xs[j] = vr[j];
         }
         if (q < n) {
+            cp[j] = a.cp[s];
             if (a.V_out) {
-                const int64_t k = t * n + a.col[s];
+                const int64_t k = t * n + (cp[j] & 0xffff);
                 if (a.v32)
                     static_cast<float2 *>(a.V_out)[k] = add2(vr[j], dl[j]);
                 else
@@ -781,7 +803,7 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
     for (int j = 0; j < kBPT; ++j) {
         const int q = base + j, s = j * th + tid;
         if (q < n) {
-            const int p = s_par[s];
+            const int p = cp[j] >> 16;
             if (kPh == 1) {
                 const float4 cs = C[s];
                 const float2 zq = make_float2(cs.z, cs.w);
@@ -820,10 +842,10 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
             if (kPh == 1) {
                 // The first child is q + 1, each next one follows the previous one's last position;
                 // the child whose subtree ends where q's ends is the last.
-                const int lq = s_rk[s] & 0xffff;
-                for (int ks = lq == s ? -1 : next_slot<kBPT>(s, th); ks >= 0;) {
-                    r = add2(r, J[ks]);
-                    const int lc = s_rk[ks] & 0xffff;
+                const int lq = s_rk[s] & 0xffff, s8 = s * kOff<kBPT>;
+                for (int ks = lq == s8 ? -1 : next_slot<kBPT>(s8, th); ks >= 0;) {
+                    r = add2(r, at8<kBPT>(J, ks));
+                    const int lc = s_rk[ks / kOff<kBPT>] & 0xffff;
                     ks = lc == lq ? -1 : next_slot<kBPT>(lc, th);
                 }
             } else {
@@ -842,8 +864,8 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
             red.z = fmaxf(red.z, v2);
             const bool under = v2 < a.v_min2, over = v2 > a.v_max2;
             red.w += (under || over) ? 1.0f : 0.0f;
-            if (under && a.bus_under) atomicAdd(&a.bus_under[a.col[s]], 1);
-            if (over && a.bus_over) atomicAdd(&a.bus_over[a.col[s]], 1);
+            if (under && a.bus_under) atomicAdd(&a.bus_under[cp[j] & 0xffff], 1);
+            if (over && a.bus_over) atomicAdd(&a.bus_over[cp[j] & 0xffff], 1);
         }
     }
     red = make_float4(warp_max(red.x), warp_max(red.y), warp_max(red.z),
@@ -884,16 +906,12 @@ TreeWork work_of(const tpf_handle *h) {
     const DeviceNet &d = h->dev;
     TreeWork w{};
     w.n = d.n;
-    w.n_ends = d.t_n_ends;
     w.vs_f = make_float2((float)h->net.vs_re, (float)h->net.vs_im);
     const float rh = (float)h->net.vs_re, ih = (float)h->net.vs_im;
     w.vs_dd = c2{{rh, (float)(h->net.vs_re - (double)rh)}, {ih, (float)(h->net.vs_im - (double)ih)}};
-    w.col = d.t_col;
-    w.end = d.t_end;
-    w.par = d.t_par;
-    w.ecnt = d.t_ecnt;
-    w.ends = d.t_ends;
-    w.kidx = d.t_kidx;
+    w.topo = d.t_topo;
+    w.cp = d.t_cp;
+    w.zf = d.t_zf;
     w.z = d.t_z;
     w.zip_hi = d.t_zip_hi;
     w.zip_lo = d.t_zip_lo;
@@ -916,10 +934,10 @@ TreeWork work_of(const tpf_handle *h) {
 size_t tree_smem(int threads, int bpt, bool zip, int phases) {
     (void)phases;
     const size_t ns = (size_t)threads * bpt;
-    // A, B, C (and the ZIP coefficients); range, parent, ends index.  The large-feeder kernel
-    // keeps only A and the indices on chip.
-    if (bpt == kTreeBigBPT) return ns * sizeof(float4) + sizeof(short) * 3 * ns;
-    return (zip ? 4 : 3) * ns * sizeof(float4) + sizeof(short) * 3 * ns;
+    // A, B, C (and the ZIP coefficients) and the range words.  The large-feeder kernel keeps only A
+    // and the range words on chip.
+    if (bpt == kTreeBigBPT) return ns * sizeof(float4) + sizeof(int) * ns;
+    return (zip ? 4 : 3) * ns * sizeof(float4) + sizeof(int) * ns;
 }
 
 // Device scratch per launch column of the large-feeder kernel.
