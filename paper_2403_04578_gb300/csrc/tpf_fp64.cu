@@ -47,14 +47,14 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
     DeviceNet &d = h->dev;
     ++d.layout_gen;
     const int n = net.n_pq;
-    cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_ends); cudaFree(d.t_z);
+    cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_z);
     cudaFree(d.t_zrow); cudaFree(d.t_yrow); cudaFree(d.t_kidx); cudaFree(d.t_zrow_f); cudaFree(d.t_z64);
     cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
     d.t_z64 = nullptr;
     d.t_topo = nullptr;
     d.t_cp = nullptr;
     d.t_zf = nullptr;
-    d.t_col = d.t_end = d.t_par = d.t_ecnt = d.t_ends = d.t_kidx = nullptr;
+    d.t_col = d.t_end = d.t_par = d.t_ecnt = d.t_kidx = nullptr;
     d.t_z = d.t_zrow = nullptr;
     d.t_yrow = d.t_zrow_f = nullptr;
     d.t_threads = d.t_bpt = 0;
@@ -67,7 +67,8 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
             const int ns = th * bpt;
             auto slot = [th, bpt](int q) { return (q % bpt) * th + q / bpt; };
             const int ph = net.phases, nb = n / ph;
-            std::vector<int> col(ns, -1), end(ns, 0), par(ns, -1), ecnt(ns, 0), ends, kidx(ns, -1);
+            std::vector<int> col(ns, -1), end(ns, 0), par(ns, -1), ecnt(ns, 0), kidx(ns, -1);
+            int n_ends = 0;  // entries of the ends lists laid out so far, in position order
             std::vector<float4> z(ns, make_float4(0.f, 0.f, 0.f, 0.f));
             std::vector<double2> z64(ph == 1 ? ns : 0, make_double2(0.0, 0.0));
             // Polyphase: row p of the branch's impedance (double-float) and admittance per slot.
@@ -82,13 +83,11 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
                 col[s] = net.dfs_col[q];
                 end[s] = net.dfs_end[q];
                 par[s] = pos_par[q] < 0 ? -1 : slot(pos_par[q]);
-                if ((int)ends.size() > 0xffff || cnt > 0x3fff) fits = false;
+                if (n_ends > 0xffff || cnt > 0x3fff) fits = false;
                 // start | count << 16 | phase << 30
-                ecnt[s] = (int)ends.size() | (cnt << 16) | ((q / nb) << 30);
-                for (int k = net.dfs_eptr[q]; k < net.dfs_eptr[q + 1]; ++k) {
-                    kidx[slot(net.dfs_ends[k])] = (int)ends.size();  // where its branch term is scattered
-                    ends.push_back(slot(net.dfs_ends[k]));
-                }
+                ecnt[s] = n_ends | (cnt << 16) | ((q / nb) << 30);
+                for (int k = net.dfs_eptr[q]; k < net.dfs_eptr[q + 1]; ++k)
+                    kidx[slot(net.dfs_ends[k])] = n_ends++;  // where its branch term is scattered
                 auto dd = [](double re, double im) {
                     const float rh = (float)re, ih = (float)im;
                     return make_float4(rh, ih, (float)(re - (double)rh), (float)(im - (double)ih));
@@ -108,24 +107,35 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
                 }
             }
             // The mixed kernel's packed words; offsets in bytes of float2 except at kTreeBigBPT, where
-            // they would not fit (bits 0-14 of the upper half, 0-15 of the lower one).
+            // they would not fit (bits 0-14 of the upper half, 0-15 of the lower one).  Of a list's
+            // positions (ascending, so the last one is the leaf before q, if the list is not empty) the
+            // leaf stays out when it belongs to q's thread: the thread takes its term from registers
+            // (bit 0 of the ends word).  Lists that the kernel finishes in a loop keep it, since it is
+            // subtracted last.
             const int unit = bpt == kTreeBigBPT ? 1 : 8;
-            std::vector<int4> topo(ns);
-            std::vector<int> cp(ns);
+            std::vector<int4> topo(ns, make_int4(0, 0, 0, 0));
+            std::vector<int> cp(ns), place(ns, -1);
             std::vector<float2> zf(ns);
+            int at = 0;
+            for (int q = 0; q < n; ++q) {
+                int cnt = net.dfs_eptr[q + 1] - net.dfs_eptr[q];
+                const bool leaf_reg = unit == 8 && q % bpt != 0 && cnt > 0 && cnt - 1 <= kTreeGather &&
+                                      net.dfs_ends[net.dfs_eptr[q + 1] - 1] == q - 1;
+                if (leaf_reg) --cnt;
+                topo[slot(q)].z = (int)((unsigned)(at * unit + (leaf_reg ? 1 : 0)) | (unsigned)cnt << 16 |
+                                        (unsigned)(q / nb) << 30);
+                for (int k = 0; k < cnt; ++k) place[slot(net.dfs_ends[net.dfs_eptr[q] + k])] = at++;
+            }
+            if ((at - 1) * unit > 0x7fff) fits = false;
             for (int s = 0; s < ns; ++s) {
                 const int q = (s % th) * bpt + s / th;
                 const int rng = ph > 1 ? end[s] : (q < n ? slot(end[s] - 1) : s) * unit;
-                const int k = kidx[s] < 0 ? -1 : kidx[s] * unit;
+                const int k = place[s] < 0 ? -1 : place[s] * unit;
                 cp[s] = (int)((unsigned)(col[s] & 0xffff) | (unsigned)par[s] << 16);
-                const unsigned ec = (unsigned)ecnt[s];
-                topo[s] = make_int4((int)((unsigned)(rng & 0xffff) | (unsigned)k << 16), cp[s],
-                                    (int)((ec & 0xffff0000u) | (ec & 0xffffu) * (unsigned)unit), 0);
+                topo[s].x = (int)((unsigned)(rng & 0xffff) | (unsigned)k << 16);
+                topo[s].y = cp[s];
                 zf[s] = make_float2(z[s].x, z[s].y);
-                if (kidx[s] * unit > 0x7fff || (int)(ec & 0xffffu) * unit > 0xffff) fits = false;
             }
-            d.t_n_ends = (int)ends.size();
-            if (ends.empty()) ends.push_back(0);
             auto up = [](auto **dst, const auto &v) -> bool {
                 using T = typename std::decay_t<decltype(v)>::value_type;
                 if (cudaMalloc((void **)dst, sizeof(T) * v.size()) != cudaSuccess) return false;
@@ -134,7 +144,7 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
             if (!fits) {
                 d.t_threads = 0;
             } else if (!up(&d.t_col, col) || !up(&d.t_end, end) || !up(&d.t_par, par) || !up(&d.t_ecnt, ecnt) ||
-                       !up(&d.t_ends, ends) || !up(&d.t_z, z) || !up(&d.t_kidx, kidx) || !up(&d.t_topo, topo) || !up(&d.t_cp, cp) ||
+                       !up(&d.t_z, z) || !up(&d.t_kidx, kidx) || !up(&d.t_topo, topo) || !up(&d.t_cp, cp) ||
                        !up(&d.t_zf, zf) ||
                        (ph == 1 && !up(&d.t_z64, z64)) || (ph > 1 && (!up(&d.t_zrow, zrow) || !up(&d.t_yrow, yrow) || !up(&d.t_zrow_f, zrow_f)))) {
                 cudaGetLastError();
@@ -296,7 +306,7 @@ void free_device(tpf_handle *h) {
     cudaFree(d.K64); cudaFree(d.W64); cudaFree(d.row_ptr); cudaFree(d.nbr); cudaFree(d.y64); cudaFree(d.y2f);
     cudaFree(d.Kr16); cudaFree(d.Ki16);
     cudaFree(d.par); cudaFree(d.ch_ptr); cudaFree(d.ch); cudaFree(d.ypar);
-    cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_ends); cudaFree(d.t_z);
+    cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_z);
     cudaFree(d.t_kidx); cudaFree(d.t_z64); cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
     cudaFree(d.zip64); cudaFree(d.t_zip_hi); cudaFree(d.t_zip_lo);
     cudaFree(d.csr_self); cudaFree(d.vs64); cudaFree(d.t_zrow); cudaFree(d.t_yrow); cudaFree(d.t_zrow_f);

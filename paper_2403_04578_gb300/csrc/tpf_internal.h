@@ -48,6 +48,7 @@ bool once_per_device(std::atomic<uint64_t> &done, F set) {
 constexpr int kTreeMaxThreads = 512;
 constexpr int kTreeBigBPT = 16;
 constexpr int kTreeBigMaxThreads = 384;  // 168 registers per thread
+constexpr int kTreeGather = 4;  // entries of an ends list that the mixed kernel gathers without a loop
 int tree_bpt(int n);  // the choice for n demand buses (TPF_TREE_BPT overrides it)
 inline int tree_threads(int n, int bpt) {
     const int t = ((n + bpt - 1) / bpt + 31) / 32 * 32;
@@ -123,12 +124,12 @@ struct DeviceNet {
     // t_bpt consecutive depth-first positions q = t_bpt k + j, stored at slot
     // s = j t_threads + k (so that a warp touches consecutive words).  Per slot: the column (-1
     // past n), the end of the subtree's position range, the parent's slot (-1 = the slack), the
-    // start and count (start | count << 16) in t_ends of the slots of the positions whose
+    // start and count (start | count << 16) in ends order of the positions whose
     // subtree range ends at q, and the double-float z of the branch to the parent
     // (re_hi, im_hi, re_lo, im_lo).
-    int t_threads = 0, t_bpt = 0, t_n_ends = 0;
-    int *t_col = nullptr, *t_end = nullptr, *t_par = nullptr, *t_ecnt = nullptr, *t_ends = nullptr;
-    int *t_kidx = nullptr;  // per slot: the index in t_ends at which its position appears, or -1
+    int t_threads = 0, t_bpt = 0;
+    int *t_col = nullptr, *t_end = nullptr, *t_par = nullptr, *t_ecnt = nullptr;
+    int *t_kidx = nullptr;  // per slot: the index in ends order at which its position appears, or -1
     float4 *t_z = nullptr;
     // What the mixed kernel reads of a slot when it sets a column up, as one 16-byte word: the range
     // word, column | parent slot << 16, the ends word (tpf_sparse.cu), 0; the second words again on

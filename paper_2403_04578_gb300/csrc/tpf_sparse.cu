@@ -45,7 +45,7 @@ namespace {
 constexpr int kMaxThreads = kTreeMaxThreads;  // so at most 8 * 512 = 4096 demand buses
 constexpr int kMaxWarps = kMaxThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kGather = 4;  // ends-list entries per position gathered without a loop
+constexpr int kGather = kTreeGather;  // ends-list entries per position gathered without a loop
 
 // One feeder's share of a launch: its network arrays (slot layout) and its tensors.
 struct TreeWork {
@@ -109,6 +109,13 @@ __device__ __forceinline__ int ends_cnt(int ec) { return (int)(((unsigned)ec >> 
 __device__ __forceinline__ int phase_of(int ec) { return (int)((unsigned)ec >> 30); }
 template <int kBPT>
 __device__ __forceinline__ int ends_start(int ec) { return (ec & 0xffff) / kOff<kBPT>; }
+// Bit 0 of the ends word (byte offsets only): the position before this one is a leaf of the
+// same thread, whose branch term, the last of those that end here, is not in the list but in the
+// thread's registers.  Half of the positions are leaves: with all of them scattered to and gathered
+// from shared memory, 131,072 columns of 1,000 buses took 10.27 ms instead of 10.12, 175,200 of 500
+// buses 5.84 instead of 5.66, and 16,384 three-phase ones of 500 buses 3.29 instead of 3.19.
+template <int kBPT>
+constexpr bool kLeafReg = kBPT != kTreeBigBPT;
 // Element of a float2 / float4 array at an offset of a word above.
 template <int kBPT>
 __device__ __forceinline__ float2 &at8(float2 *p, int off) {
@@ -400,10 +407,10 @@ __device__ __forceinline__ c2 anchor_dd(const TreeWork &a, float4 *A, float4 *B,
         if (k >= 0) at16<kBPT>(A, k) = B[s];
     }
     __syncthreads();
-    // Inclusive prefix sums of E_q = x_q - (x_b of every b whose range ends at q), into B.
-    run = c2{{0.0f, 0.0f}, {0.0f, 0.0f}};
+    // E_q = x_q - (x_b of every b whose range ends at q) into B, descending j (position q - 1 of the
+    // thread still holds its x), then the inclusive prefix sums.
 #pragma unroll 1
-    for (int j = 0; j < kBPT; ++j) {
+    for (int j = kBPT - 1; j >= 0; --j) {
         const int q = base + j, s = j * th + tid;
         if (q < n) {
             int ec = ecnt[0];  // ecnt[j] by selects: the array stays in registers
@@ -411,10 +418,20 @@ __device__ __forceinline__ c2 anchor_dd(const TreeWork &a, float4 *A, float4 *B,
             for (int i = 1; i < kBPT; ++i)
                 if (j == i) ec = ecnt[i];
             const int st = ends_start<kBPT>(ec), cnt = ends_cnt(ec);
+            if (cnt == 0 && !(kLeafReg<kBPT> && (ec & 1))) continue;
             c2 e = unpack(B[s]);
 #pragma unroll 1
             for (int k = 0; k < cnt; ++k) e = cqsub(e, unpack(A[st + k]));
-            run = cqadd(run, e);
+            if (kLeafReg<kBPT> && (ec & 1)) e = cqsub(e, unpack(B[s - th]));
+            B[s] = pack(e);
+        }
+    }
+    run = c2{{0.0f, 0.0f}, {0.0f, 0.0f}};
+#pragma unroll 1
+    for (int j = 0; j < kBPT; ++j) {
+        const int s = j * th + tid;
+        if (base + j < n) {
+            run = cqadd(run, unpack(B[s]));
             B[s] = pack(run);
         }
     }
@@ -451,7 +468,11 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
     float4 *const A = tsm;       // [ns] double-float prefix sums (anchor); float2 P and X in the sweeps
     float4 *const big = kBig ? g.scratch + (size_t)blockIdx.x * (kZip ? 3 : 2) * ns : nullptr;
     float4 *const B = kBig ? big : tsm + ns;  // [ns] V_ref (anchor input), x (anchor), then D = BFS(V_ref) - V_ref
-    float4 *const C = kBig ? big + ns : tsm + 2 * ns;  // [ns] (S_hi, z_hi) of each position
+    // S_hi and z_hi of each position, apart: a sweep reads each once, 8 bytes a lane without conflicts
+    // (side by side in a float4 each read moved the other one too: 10.44 against 10.27 ms on 131,072
+    // columns of 1,000 buses; the shared-memory pipe was at 75 % of its peak).
+    float2 *const Sv = reinterpret_cast<float2 *>(kBig ? big + ns : tsm + 2 * ns);  // [ns]
+    float2 *const Zv = Sv + ns;                                                     // [ns]
     float4 *const Zs = kBig ? big + 2 * ns : tsm + 3 * ns;  // [ns] ZIP coefficients (kZip only)
     // [ns] range words.  Bits 0-15, the subtree's range [q, end_q): one phase, the slot of its last
     // position end_q - 1 (the slot itself for a leaf); polyphase, end_q.  Bits 16-31: where the
@@ -498,7 +519,8 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
             }
             zh = a.zf[s];
         }
-        C[s] = make_float4(sh.x, sh.y, zh.x, zh.y);
+        Sv[s] = sh;
+        Zv[s] = zh;
         B[s] = make_float4(sl.x, sl.y, 0.0f, 0.0f);  // S_lo until the first anchor replaces it by D
         if (kZip) Zs[s] = q < n ? a.zip_hi[s] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
@@ -582,7 +604,7 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
                     float2 slo = make_float2(0.0f, 0.0f);
                     if (q < n && !a.s32) {
                         const double2 sv = S64[a.cp[s] & 0xffff];
-                        const float4 cs = C[s];
+                        const float2 cs = Sv[s];
                         slo = make_float2(__double2float_rn(sv.x - (double)cs.x), __double2float_rn(sv.y - (double)cs.y));
                     }
                     B[s] = make_float4(slo.x, slo.y, 0.0f, 0.0f);
@@ -595,7 +617,8 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
                 const f2 re = two_sum(vr[j].x, dl[j].x), im = two_sum(vr[j].y, dl[j].y);
                 vr[j] = make_float2(re.h, im.h);
                 dl[j] = make_float2(re.l, im.l);
-                const float4 cs = C[s], b = B[s];  // b = (S_lo, -)
+                const float2 cs = Sv[s];
+                const float4 b = B[s];  // (S_lo, -)
                 A[s] = make_float4(cs.x, cs.y, 0.0f, 0.0f);
                 B[s] = make_float4(re.h, im.h, b.x, b.y);
             }
@@ -626,17 +649,17 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
             if (anchored) {
 #pragma unroll
                 for (int j = 0; j < kBPT; ++j) {
-                    const float4 cs = C[j * th + tid];
+                    const float2 cs = Sv[j * th + tid];
                     const float4 al = kZip ? Zs[j * th + tid] : make_float4(1.0f, 0.0f, 0.0f, 0.0f);
-                    run = add2(run, demand_change<kZip>(vr[j], dl[j], make_float2(cs.x, cs.y), al));
+                    run = add2(run, demand_change<kZip>(vr[j], dl[j], cs, al));
                     loc[j] = run;  // positions past n have S = 0 and add nothing
                 }
             } else {
 #pragma unroll
                 for (int j = 0; j < kBPT; ++j) {
-                    const float4 cs = C[j * th + tid];
+                    const float2 cs = Sv[j * th + tid];
                     const float4 al = kZip ? Zs[j * th + tid] : make_float4(1.0f, 0.0f, 0.0f, 0.0f);
-                    run = add2(run, demand_current<kZip>(vr[j], make_float2(cs.x, cs.y), al));
+                    run = add2(run, demand_current<kZip>(vr[j], cs, al));
                     loc[j] = run;
                 }
             }
@@ -683,8 +706,7 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
                         float2 L = ls == s * kOff<kBPT> ? loc[j] : at8<kBPT>(P, ls);
                         if (j) L = sub2(L, loc[j - 1]);
                         else if (q > 0) L = sub2(L, P[(kBPT - 1) * th + tid - 1]);
-                        const float4 cs = C[s];
-                        xq = cmul2(make_float2(cs.z, cs.w), L);
+                        xq = cmul2(Zv[s], L);
                     } else {
                         // x = sum over phases p' of Z[p][p'] L_{p'}
                         const int p = phase_of(ecnt[j]), qb = q - p * a.nbp, eb = (rk & 0xffff) - p * a.nbp;
@@ -707,16 +729,18 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
             // Path sums: prefix sums of E_q = x_q - (x_b of every b whose subtree range ends at
             // q).  Up to kGather entries per position unrolled and predicated; longer lists (rare:
             // a drop of more than kGather levels between neighbouring positions) finish in a loop.
+            // Descending j: loc[j - 1] still holds x of position q - 1.
             bool longer = false;
 #pragma unroll
-            for (int j = 0; j < kBPT; ++j) {
+            for (int j = kBPT - 1; j >= 0; --j) {
                 // The count sits above the start: count > k is word >= (k + 1) << 16.
-                const int st = ecnt[j] & 0xffff, ec = kPh > 1 ? ecnt[j] & 0x3fffffff : ecnt[j];
+                const int st = ecnt[j] & (kOff<kBPT> == 1 ? 0xffff : 0xfff8), ec = kPh > 1 ? ecnt[j] & 0x3fffffff : ecnt[j];
                 float2 e = loc[j];
                 const float2 *Xs = &at8<kBPT>(X, st);
 #pragma unroll
                 for (int k = 0; k < kGather; ++k)
                     if (ec >= (k + 1) << 16) e = sub2(e, Xs[k]);
+                if (kLeafReg<kBPT> && j && (ecnt[j] & 1)) e = sub2(e, loc[j - 1]);
                 longer |= ec >= (kGather + 1) << 16;
                 loc[j] = e;
             }
@@ -805,8 +829,7 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
         if (q < n) {
             const int p = cp[j] >> 16;
             if (kPh == 1) {
-                const float4 cs = C[s];
-                const float2 zq = make_float2(cs.z, cs.w);
+                const float2 zq = Zv[s];
                 const float inv = __fdividef(1.0f, abs2(zq));
                 const float2 yk = make_float2(zq.x * inv, -zq.y * inv);
                 J[s] = cmul2(yk, sub2(p >= 0 ? X[p] : x_slack, xs[j]));
@@ -834,8 +857,7 @@ __global__ void __maxnreg__(kBPT == 16 ? 168 : (kBPT == 8 ? 128 : (kBPT == 4 && 
     for (int j = 0; j < kBPT; ++j) {
         const int q = base + j, s = j * th + tid;
         if (q < n) {
-            const float4 cs = C[s];
-            const float2 sh = make_float2(cs.x, cs.y);
+            const float2 sh = Sv[s];
             const float4 al = kZip ? Zs[s] : make_float4(1.0f, 0.0f, 0.0f, 0.0f);
             float2 r = anchored ? demand_change<kZip>(vr[j], dl[j], sh, al) : demand_current<kZip>(vr[j], sh, al);
             r = sub2(r, J[s]);
