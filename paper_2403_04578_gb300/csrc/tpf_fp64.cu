@@ -1,12 +1,14 @@
 // Device buffers of a handle and the plain double-precision solve path.
 //
 // The FP64 path is Algorithm 1 in its direct form, V_{k+1} = K conj(S ./ V_k) + W (Eq. 2 and
-// Eq. 12), with per-column stopping.  Each sweep is one kernel over (64-bus x 32-column) output
-// tiles: the tile's injections conj(S ./ V) are formed from V_k in shared memory chunk by chunk
-// (the Hadamard step of Algorithm 1), multiplied by the matching K tile with FP64 FMAs, W is
-// added and the per-column max |V_{k+1} - V_k| is folded in with an atomic max.  GB300 runs FP64
-// at 1/64 of its FP32 rate, so this path is FP64-pipe bound; it is the reference point for the
-// mixed-precision path.
+// Eq. 12), with per-column stopping.  GB300 runs FP64 at 1/64 of its FP32 rate, so the sweeps of all but
+// the smallest networks go to the tensor cores in exact fixed point (tpf_fixed.cu, which also has the
+// rule).  Here each sweep is one kernel over (64-bus x 32-column) output tiles: the tile's injections
+// conj(S ./ V) are formed from V_k in shared memory chunk by chunk (the Hadamard step of Algorithm 1),
+// multiplied by the matching K tile with FP64 FMAs, W is added and the per-column max |V_{k+1} - V_k| is
+// folded in with an atomic max.  It also serves the allocation-free solve, which has no room for digit
+// planes.
+#include <algorithm>
 #include <cstdio>
 #include <type_traits>
 #include <math_constants.h>
@@ -170,6 +172,15 @@ tpf_status upload_network(tpf_handle *h) {
     TPF_CK(cudaMalloc(&d.y64, sizeof(double) * 2 * (nnz > 0 ? nnz : 1)));
     TPF_CK(cudaMalloc(&d.y2f, sizeof(float4) * (nnz > 0 ? nnz : 1)));
     TPF_CK(cudaMemcpy(d.row_ptr, net.row_ptr.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice));
+    {
+        std::vector<int> order(n);
+        for (int i = 0; i < n; ++i) order[i] = i;
+        std::stable_sort(order.begin(), order.end(), [&net](int a, int b) {
+            return net.row_ptr[a + 1] - net.row_ptr[a] < net.row_ptr[b + 1] - net.row_ptr[b];
+        });
+        TPF_CK(cudaMalloc(&d.row_order, sizeof(int) * n));
+        TPF_CK(cudaMemcpy(d.row_order, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
+    }
     if (nnz > 0) {
         TPF_CK(cudaMemcpy(d.nbr, net.nbr.data(), sizeof(int) * nnz, cudaMemcpyHostToDevice));
         TPF_CK(cudaMemcpy(d.y64, net.y.data(), sizeof(double) * 2 * nnz, cudaMemcpyHostToDevice));
@@ -303,8 +314,8 @@ tpf_status set_zip(tpf_handle *h, const double *alpha) {
 
 void free_device(tpf_handle *h) {
     DeviceNet &d = h->dev;
-    cudaFree(d.K64); cudaFree(d.W64); cudaFree(d.row_ptr); cudaFree(d.nbr); cudaFree(d.y64); cudaFree(d.y2f);
-    cudaFree(d.Kr16); cudaFree(d.Ki16);
+    cudaFree(d.K64); cudaFree(d.W64); cudaFree(d.row_ptr); cudaFree(d.nbr); cudaFree(d.row_order); cudaFree(d.y64); cudaFree(d.y2f);
+    cudaFree(d.Kr16); cudaFree(d.Ki16); cudaFree(d.Kd16);
     cudaFree(d.par); cudaFree(d.ch_ptr); cudaFree(d.ch); cudaFree(d.ypar);
     cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_z);
     cudaFree(d.t_kidx); cudaFree(d.t_z64); cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
@@ -314,7 +325,7 @@ void free_device(tpf_handle *h) {
     Workspace &w = h->ws;
     cudaFree(w.Vhi); cudaFree(w.Vlo); cudaFree(w.Shi); cudaFree(w.Slo); cudaFree(w.Rr16); cudaFree(w.Ri16);
     cudaFree(w.RefHi); cudaFree(w.RefLo); cudaFree(w.dprev);
-    cudaFree(w.Valt); cudaFree(w.delta_bits); cudaFree(w.delta64); cudaFree(w.iters); cudaFree(w.flags);
+    cudaFree(w.Valt); cudaFree(w.fx_buf); cudaFree(w.delta_bits); cudaFree(w.delta64); cudaFree(w.iters); cudaFree(w.flags);
     cudaFree(w.rexp); cudaFree(w.tile_active); cudaFree(w.counters);
     if (w.counters_host) cudaFreeHost(w.counters_host);
     cudaFree(w.S_dev); cudaFree(w.V_dev); cudaFree(w.it_dev); cudaFree(w.mm_dev); cudaFree(w.tree_scratch);
@@ -335,7 +346,7 @@ tpf_status ensure_workspace(tpf_handle *h, int64_t cols, int kind) {
     const bool have_fp64 = w.Valt != nullptr;
     if (w.counters == nullptr) {
         TPF_CK(cudaMalloc(&w.counters, sizeof(int) * 8));
-        TPF_CK(cudaMallocHost(&w.counters_host, sizeof(int) * 8));
+        TPF_CK(cudaMallocHost(&w.counters_host, sizeof(int) * 16));
         TPF_CK(cudaMemset(w.counters, 0, sizeof(int) * 8));
     }
     if (cols <= w.cap_cols && (mixed ? have_mixed : (fp64 ? have_fp64 : true))) return TPF_OK;
@@ -525,27 +536,33 @@ __global__ void f64_decide(int64_t T, double tol, int max_iter, int *flags, int 
     }
 }
 
-// Copy the final iterate into V (when it sits in the second buffer), write the iteration counts
+// Copy the final iterate into V (when there is a second buffer and it sits there), write the iteration counts
 // and the FP64 power mismatch max_i |V_i conj(sum_j y_ij (V_i - V_j)) + S_i|.
 __global__ void f64_finish(int64_t T, int n, int max_iter, const int *__restrict__ flags,
                            const int *__restrict__ it_state, double2 *V, const double2 *__restrict__ Valt,
                            const double2 *__restrict__ S, const int *__restrict__ row_ptr,
-                           const int *__restrict__ nbr, const double2 *__restrict__ y,
-                           const int *__restrict__ self, const double2 *__restrict__ vs,
+                           const int *__restrict__ nbr, const int *__restrict__ order,
+                           const double2 *__restrict__ y, const int *__restrict__ self, const double2 *__restrict__ vs,
                            const double *__restrict__ zip, int32_t *iters_out, double *mismatch_out) {
     const int lane = threadIdx.x & 31;
     const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (t >= T) return;
     const int updates = it_state[t];
-    if (updates & 1) {
+    if (Valt && (updates & 1)) {
         for (int i = lane; i < n; i += 32) V[t * n + i] = Valt[t * n + i];
     }
     __syncwarp();
     if (lane == 0 && iters_out) iters_out[t] = (flags[t] & kDone) ? updates : -max_iter;
     if (!mismatch_out) return;
-    double worst = 0.0;
+    // worst2: the largest square of the mismatches, where a square neither underflows nor overflows; worst:
+    // the others and those of ZIP loads.  With a hypot per bus, and the buses in their own order, 8,760
+    // columns of 199 buses took 273 us instead of 197.
+    double worst = 0.0, worst2 = 0.0;
     const double2 *v = V + t * n;
-    for (int i = lane; i < n; i += 32) {
+    for (int k = lane; k < n; k += 32) {
+        // Buses by the length of their lists, so that the lanes of a warp loop alike: the FP64 pipe takes
+        // an instruction's time whatever the number of lanes that need it.
+        const int i = order[k];
         double2 vi = v[i];
         double2 acc = make_double2(0.0, 0.0);
         for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
@@ -572,10 +589,17 @@ __global__ void f64_finish(int64_t T, int n, int max_iter, const int *__restrict
             // V_i conj(acc) + S_i
             double mr = vi.x * acc.x + vi.y * acc.y + s.x;
             double mi = vi.y * acc.x - vi.x * acc.y + s.y;
+            const double m2 = fma(mr, mr, mi * mi);
+            if (m2 > 1e-280 && m2 < 1e280) {  // neither rounds away nor overflows; false for NaN
+                worst2 = m2 > worst2 ? m2 : worst2;
+                continue;
+            }
             m = hypot(mr, mi);
         }
         if (!(m <= worst)) worst = m;
     }
+    worst2 = sqrt(worst2);
+    if (worst2 > worst) worst = worst2;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         double other = __shfl_xor_sync(0xffffffffu, worst, o);
@@ -590,48 +614,55 @@ tpf_status solve_fp64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t 
                       const tpf_opts &o, cudaStream_t st) {
     tpf_status rs = ensure_dense(h);
     if (rs != TPF_OK) return rs;
-    rs = ensure_workspace(h, T, kWsFp64);
+    const bool fixed = use_fixed(h->dev.n, T);
+    rs = ensure_workspace(h, T, fixed ? kWsState : kWsFp64);
     if (rs != TPF_OK) return rs;
     Workspace &w = h->ws;
     const int n = h->dev.n;
     const int64_t cols = round_up(T, kTileN);
-    int64_t launches = 0;
-    KernelTimer timer(o.profile != 0, st);
-    TPF_CK(cudaMemsetAsync(w.counters, 0, sizeof(int) * 8, st));
-    {
-        int64_t work = cols > T * n ? cols : T * n;
-        f64_init<<<(unsigned)((work + 255) / 256), 256, 0, st>>>(T, cols, n, o.start == TPF_START_FLAT,
-                                                                  (double2 *)V, w.flags, w.iters, w.delta64);
-        ++launches;
-    }
-    TPF_CK(cudaGetLastError());
-    double2 *buf[2] = {(double2 *)V, (double2 *)w.Valt};
-    const dim3 grid((unsigned)((T + F64_BN - 1) / F64_BN), (n + F64_BM - 1) / F64_BM);
+    int64_t launches = 0, gemms = 0, gemm_cols = 0;
     int sweeps = 0;
-    int64_t active = T, gemm_cols = 0;
-    for (int k = 0; k < o.max_iter; ++k) {
-        timer.begin(KernelTimer::kGemm);
-        f64_sweep<<<grid, 256, 0, st>>>((const double2 *)h->dev.K64, (const double2 *)h->dev.W64, (const double2 *)S,
-                                        buf[k & 1], buf[(k + 1) & 1], n, T, w.flags, w.delta64, h->dev.zip64);
-        timer.end();
-        gemm_cols += active;
-        TPF_CK(cudaMemsetAsync(w.counters, 0, sizeof(int) * 4, st));
-        timer.begin(KernelTimer::kResidual);
-        f64_decide<<<(unsigned)((T + 255) / 256), 256, 0, st>>>(T, o.tol, o.max_iter, w.flags, w.iters, w.delta64,
-                                                                w.counters);
-        timer.end();
-        launches += 2;
+    KernelTimer timer(o.profile != 0, st);
+    if (fixed) {
+        rs = solve_fixed(h, T, S, V, o, st, timer, &sweeps, &launches, &gemms, &gemm_cols);
+        if (rs != TPF_OK) return rs;
+    } else {
+        TPF_CK(cudaMemsetAsync(w.counters, 0, sizeof(int) * 8, st));
+        {
+            int64_t work = cols > T * n ? cols : T * n;
+            f64_init<<<(unsigned)((work + 255) / 256), 256, 0, st>>>(T, cols, n, o.start == TPF_START_FLAT,
+                                                                      (double2 *)V, w.flags, w.iters, w.delta64);
+            ++launches;
+        }
         TPF_CK(cudaGetLastError());
-        ++sweeps;
-        TPF_CK(cudaMemcpyAsync(w.counters_host, w.counters, sizeof(int) * 4, cudaMemcpyDeviceToHost, st));
-        TPF_CK(cudaStreamSynchronize(st));
-        active = w.counters_host[kCntActive];
-        if (active == 0) break;
+        double2 *buf[2] = {(double2 *)V, (double2 *)w.Valt};
+        const dim3 grid((unsigned)((T + F64_BN - 1) / F64_BN), (n + F64_BM - 1) / F64_BM);
+        int64_t active = T;
+        for (int k = 0; k < o.max_iter; ++k) {
+            timer.begin(KernelTimer::kGemm);
+            f64_sweep<<<grid, 256, 0, st>>>((const double2 *)h->dev.K64, (const double2 *)h->dev.W64, (const double2 *)S,
+                                            buf[k & 1], buf[(k + 1) & 1], n, T, w.flags, w.delta64, h->dev.zip64);
+            timer.end();
+            gemm_cols += active;
+            TPF_CK(cudaMemsetAsync(w.counters, 0, sizeof(int) * 4, st));
+            timer.begin(KernelTimer::kResidual);
+            f64_decide<<<(unsigned)((T + 255) / 256), 256, 0, st>>>(T, o.tol, o.max_iter, w.flags, w.iters, w.delta64,
+                                                                    w.counters);
+            timer.end();
+            launches += 2;
+            TPF_CK(cudaGetLastError());
+            ++sweeps;
+            TPF_CK(cudaMemcpyAsync(w.counters_host, w.counters, sizeof(int) * 4, cudaMemcpyDeviceToHost, st));
+            TPF_CK(cudaStreamSynchronize(st));
+            active = w.counters_host[kCntActive];
+            if (active == 0) break;
+        }
+        gemms = sweeps;
     }
     timer.begin(KernelTimer::kOther);
     f64_finish<<<(unsigned)((T * 32 + 255) / 256), 256, 0, st>>>(
-        T, n, o.max_iter, w.flags, w.iters, (double2 *)V, (const double2 *)w.Valt, (const double2 *)S,
-        h->dev.row_ptr, h->dev.nbr, (const double2 *)h->dev.y64, h->dev.csr_self, (const double2 *)h->dev.vs64,
+        T, n, o.max_iter, w.flags, w.iters, (double2 *)V, fixed ? nullptr : (const double2 *)w.Valt, (const double2 *)S,
+        h->dev.row_ptr, h->dev.nbr, h->dev.row_order, (const double2 *)h->dev.y64, h->dev.csr_self, (const double2 *)h->dev.vs64,
         h->dev.zip64, iters, mismatch);
     timer.end();
     ++launches;
@@ -641,7 +672,7 @@ tpf_status solve_fp64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t 
     h->stats.sweeps = sweeps;
     h->stats.kernel_launches = launches;
     h->stats.converged = w.counters_host[kCntConverged];
-    h->stats.gemm_launches = sweeps;
+    h->stats.gemm_launches = gemms;
     h->stats.gemm_columns = gemm_cols;
     h->stats.gemm_ms = timer.total_ms(KernelTimer::kGemm);
     h->stats.residual_ms = timer.total_ms(KernelTimer::kResidual);
@@ -738,7 +769,7 @@ extern "C" tpf_status tpf_solve_fp64_noalloc(int n, const void *K_dev, const voi
     }
     f64_finish<<<(unsigned)((T * 32 + 255) / 256), 256, 0, st>>>(T, n, max_iter, flags, iters, (double2 *)V_dev,
                                                                  Valt, (const double2 *)S_dev, nullptr, nullptr,
-                                                                 nullptr, nullptr, nullptr, nullptr, iters_dev,
+                                                                 nullptr, nullptr, nullptr, nullptr, nullptr, iters_dev,
                                                                  nullptr);
     TPF_CK(cudaGetLastError());
     TPF_CK(cudaMemcpyAsync(host_counters, counters, sizeof(int) * 8, cudaMemcpyDeviceToHost, st));

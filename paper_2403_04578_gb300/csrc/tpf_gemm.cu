@@ -335,13 +335,14 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-// A [rows][inner] 16-bit matrix read in (128 rows x 64 elements) boxes, 128-byte swizzle.
-bool make_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, bool bf16) {
+// A [rows][inner] 16-bit matrix read in (box_rows x 64 elements) boxes, 128-byte swizzle.
+bool make_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, bool bf16,
+              uint32_t box_rows = kTileM) {
     auto fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {inner, rows};
     cuuint64_t strides[1] = {inner * 2};
-    cuuint32_t box[2] = {(cuuint32_t)kChunkK, (cuuint32_t)kTileM};
+    cuuint32_t box[2] = {(cuuint32_t)kChunkK, box_rows};
     cuuint32_t estr[2] = {1, 1};
     return fn(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -352,6 +353,10 @@ bool make_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows,
 
 bool make_bf16_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows) {
     return make_map(map, base, inner, rows, true);
+}
+
+bool make_f16_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, uint32_t box_rows) {
+    return make_map(map, base, inner, rows, false, box_rows);
 }
 
 bool make_f64_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, uint32_t box_inner,

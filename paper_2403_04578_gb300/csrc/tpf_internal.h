@@ -115,6 +115,7 @@ struct DeviceNet {
     double *K64 = nullptr;   // complex [n][n]
     double *W64 = nullptr;   // complex [n]
     int *row_ptr = nullptr, *nbr = nullptr;
+    int *row_order = nullptr;  // the demand buses by the length of their neighbour lists
     double *y64 = nullptr;   // complex [nnz]
     float4 *y2f = nullptr;   // double-float complex admittance (re_hi, im_hi, re_lo, im_lo) [nnz]
     bool radial = false;
@@ -156,6 +157,8 @@ struct DeviceNet {
     // Mixed path: fp16 planes of K * 2^k_exp, [n_pad][n_pad], zero padded
     void *Kr16 = nullptr, *Ki16 = nullptr;
     int k_exp = 0;
+    // FP64 path on the tensor cores: fp16 digit planes of K (Re, then Im), [2][7][n_pad][n_pad]
+    void *Kd16 = nullptr;
     // Incremented whenever the sparse layout or the ZIP coefficients are replaced: a prepared
     // batch (tpf_batch) that captured the old device arrays then refuses to launch.
     int layout_gen = 0;
@@ -175,6 +178,9 @@ struct Workspace {
     unsigned int *dprev = nullptr;        // float bits of the step before the last (mixed)
     // FP64 path: second V buffer, complex128 [cols][n]
     double *Valt = nullptr;
+    // FP64 path on the tensor cores: digit planes of the injections, their orders, column lists
+    void *fx_buf = nullptr;
+    size_t fx_bytes = 0;
     // per-column state
     unsigned int *delta_bits = nullptr;   // float bits (mixed) of the last max|dV|
     unsigned long long *delta64 = nullptr;// double bits (FP64 path)
@@ -295,6 +301,11 @@ tpf_status ensure_workspace(tpf_handle *h, int64_t cols, int kind);
 // The two solve paths.  Return TPF_OK / TPF_ENOCONV / errors.
 tpf_status solve_fp64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t *iters,
                       double *mismatch, const tpf_opts &o, cudaStream_t st);
+// The sweeps of the FP64 dense path in fixed point on the tensor cores (tpf_fixed.cu), V updated in
+// place; use_fixed says which sizes take it.
+bool use_fixed(int n, int64_t T);
+tpf_status solve_fixed(tpf_handle *h, int64_t T, const void *S, void *V, const tpf_opts &o, cudaStream_t st,
+                       KernelTimer &timer, int *sweeps, int64_t *launches, int64_t *gemms, int64_t *gemm_cols);
 tpf_status solve_mixed(tpf_handle *h, int64_t T, const void *S, void *V, int32_t *iters,
                        double *mismatch, const tpf_opts &o, cudaStream_t st);
 tpf_status solve_sparse(tpf_handle *h, int64_t T, const void *S, void *V, int32_t *iters,
