@@ -66,24 +66,16 @@ __device__ __forceinline__ c2 load_current_dd(c2 s, c2 v) {
     return {dd_mul(nr, inv), dd_mul(ni, inv)};
 }
 
-// hi[k] + lo[k] as a normalised double-float (lo == nullptr reads as zero).
-__device__ __forceinline__ c2 load_c2(const float2 *hi, const float2 *lo, int64_t k) {
-    float2 a = hi[k];
-    if (!lo) return {{a.x, 0.0f}, {a.y, 0.0f}};
-    float2 b = lo[k];
-    return {two_sum(a.x, b.x), two_sum(a.y, b.y)};
-}
-
-// rho_i in double-float for bus i of the column whose V planes start at vh / vl, any network:
+// rho_i in double-float for bus i (load s) of the column whose FP32 voltages start at vh, any network:
 // (Y v)_i = sum_j y_ij (V_i - V_j) over the branches at bus i, V_slack = vs.
-__device__ __forceinline__ c2 residual_dd(int i, const float2 *vh, const float2 *vl, const float2 *sh,
-                                          const float2 *sl, const int *row_ptr, const int *nbr, const float4 *y,
-                                          c2 vs) {
-    c2 v = load_c2(vh, vl, i);
-    c2 acc = load_current_dd(load_c2(sh, sl, i), v);
+__device__ __forceinline__ c2 residual_dd(int i, const float2 *vh, c2 s, const int *row_ptr, const int *nbr,
+                                          const float4 *y, c2 vs) {
+    c2 v = {{vh[i].x, 0.0f}, {vh[i].y, 0.0f}};
+    c2 acc = load_current_dd(s, v);
     for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
         int j = nbr[e];
-        c2 vj = j >= 0 ? load_c2(vh, vl, j) : vs;
+        c2 vj = vs;
+        if (j >= 0) vj = c2{{vh[j].x, 0.0f}, {vh[j].y, 0.0f}};
         float4 ye = y[e];
         c2 yy = {{ye.x, ye.z}, {ye.y, ye.w}};
         acc = c_add(acc, c_mul(yy, c_sub(v, vj)));
@@ -148,28 +140,29 @@ __device__ __forceinline__ float pow2f(int e) {
     return __int_as_float((127 + e) << 23);
 }
 
-// Arguments of the per-sweep residual kernel.
+// Arguments of the per-sweep residual kernels.
 struct PrologueArgs {
-    int64_t cols;
+    int64_t cols, T;
     int n, n_pad, sweep, max_iter;
     float tol, switch_tol;
     float2 vs_f;
     c2 vs_dd;
-    float2 *Vhi, *Vlo;
-    const float2 *Shi, *Slo;
+    const double2 *S64, *V0;  // the caller's S, and V_0 (null: flat start)
+    float2 *Vhi, *Vlo, *Shi;
     float2 *RefHi, *RefLo;
     const int *row_ptr, *nbr;
     const float4 *y;
     int *flags, *iters, *rexp, *tile_active, *counters;
     unsigned *delta, *dprev;
     int given;  // the solve started from a given V_0: anchor every column at sweep 0
-    int radial;
-    const int *par, *ch_ptr, *ch;
-    const float2 *ypar;
+    const int4 *topo;     // radial feeders: per-bus words (tpf_residual.cu), else null
+    const int2 *inner;    // the buses with children (n_inner)
+    int n_inner;
+    const float4 *ypar4;  // and the double-float admittance of each bus's branch to its parent
     __half *Rr, *Ri;
 };
 
-// Launch the residual kernel of one sweep (tpf_residual.cu).
+// Launch the residual kernel of one sweep (tpf_residual.cu); sweep 0 also sets up the columns' state.
 tpf_status launch_residual(const PrologueArgs &a, cudaStream_t st);
 // Final outputs of a solve: V (complex128 [T][n]), iteration counts, mismatch, and the converged
 // columns counted per 128-column tile into tile_done (zeroed by the caller).

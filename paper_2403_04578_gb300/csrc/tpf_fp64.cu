@@ -10,6 +10,7 @@
 // planes.
 #include <algorithm>
 #include <cstdio>
+#include <cstring>
 #include <type_traits>
 #include <math_constants.h>
 
@@ -207,18 +208,35 @@ tpf_status upload_network(tpf_handle *h) {
         if (vs.empty()) vs = {net.vs_re, net.vs_im};
         TPF_CK(cudaMemcpy(d.vs64, vs.data(), sizeof(double) * 2 * net.phases, cudaMemcpyHostToDevice));
     }
-    if (net.radial && net.phases == 1) {
-        const int nch = net.ch_ptr[n];
-        std::vector<float2> yp(n);
-        for (int i = 0; i < n; ++i) yp[i] = make_float2((float)net.ypar[2 * i], (float)net.ypar[2 * i + 1]);
-        TPF_CK(cudaMalloc(&d.par, sizeof(int) * n));
-        TPF_CK(cudaMalloc(&d.ch_ptr, sizeof(int) * (n + 1)));
-        TPF_CK(cudaMalloc(&d.ch, sizeof(int) * (nch > 0 ? nch : 1)));
-        TPF_CK(cudaMalloc(&d.ypar, sizeof(float2) * n));
-        TPF_CK(cudaMemcpy(d.par, net.par.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
-        TPF_CK(cudaMemcpy(d.ch_ptr, net.ch_ptr.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice));
-        if (nch > 0) TPF_CK(cudaMemcpy(d.ch, net.ch.data(), sizeof(int) * nch, cudaMemcpyHostToDevice));
-        TPF_CK(cudaMemcpy(d.ypar, yp.data(), sizeof(float2) * n, cudaMemcpyHostToDevice));
+    if (net.radial && net.phases == 1 && d.n_pad <= 2048) {
+        std::vector<int4> topo(n);
+        std::vector<float4> yp(n);
+        std::vector<int> place(n, -1);
+        std::vector<int2> inner;
+        for (int k = 0; k < net.ch_ptr[n]; ++k) place[net.ch[k]] = k;
+        for (int i = 0; i < n; ++i) {
+            const float rh = (float)net.ypar[2 * i], ih = (float)net.ypar[2 * i + 1];
+            for (int e = net.row_ptr[i]; e < net.row_ptr[i + 1]; ++e)
+                if (net.nbr[e] == net.par[i]) {
+                    const double re = net.y[2 * e], im = net.y[2 * e + 1];
+                    yp[i] = make_float4((float)re, (float)im, (float)(re - (double)(float)re), (float)(im - (double)(float)im));
+                }
+            topo[i].x = (int)((unsigned)(net.par[i] & 0xffff) | (unsigned)place[i] << 16);
+            topo[i].y = 0;
+            const int kids = net.ch_ptr[i + 1] - net.ch_ptr[i];
+            if (kids > 0) inner.push_back(make_int2((int)((unsigned)i | (unsigned)kids << 16), net.ch_ptr[i]));
+            memcpy(&topo[i].z, &rh, sizeof(float));
+            memcpy(&topo[i].w, &ih, sizeof(float));
+        }
+        std::stable_sort(inner.begin(), inner.end(),
+                         [](int2 a, int2 b) { return ((unsigned)a.x >> 16) > ((unsigned)b.x >> 16); });
+        d.r_n_inner = (int)inner.size();
+        TPF_CK(cudaMalloc(&d.r_inner, sizeof(int2) * (inner.size() + 1)));
+        TPF_CK(cudaMemcpy(d.r_inner, inner.data(), sizeof(int2) * inner.size(), cudaMemcpyHostToDevice));
+        TPF_CK(cudaMalloc(&d.r_topo, sizeof(int4) * n));
+        TPF_CK(cudaMalloc(&d.r_ypar, sizeof(float4) * n));
+        TPF_CK(cudaMemcpy(d.r_topo, topo.data(), sizeof(int4) * n, cudaMemcpyHostToDevice));
+        TPF_CK(cudaMemcpy(d.r_ypar, yp.data(), sizeof(float4) * n, cudaMemcpyHostToDevice));
     }
     if (net.radial) {
         const tpf_status rs = layout_tree(h, tree_bpt(n));
@@ -316,18 +334,19 @@ void free_device(tpf_handle *h) {
     DeviceNet &d = h->dev;
     cudaFree(d.K64); cudaFree(d.W64); cudaFree(d.row_ptr); cudaFree(d.nbr); cudaFree(d.row_order); cudaFree(d.y64); cudaFree(d.y2f);
     cudaFree(d.Kr16); cudaFree(d.Ki16); cudaFree(d.Kd16);
-    cudaFree(d.par); cudaFree(d.ch_ptr); cudaFree(d.ch); cudaFree(d.ypar);
+    cudaFree(d.r_topo); cudaFree(d.r_inner); cudaFree(d.r_ypar);
     cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_z);
     cudaFree(d.t_kidx); cudaFree(d.t_z64); cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
     cudaFree(d.zip64); cudaFree(d.t_zip_hi); cudaFree(d.t_zip_lo);
     cudaFree(d.csr_self); cudaFree(d.vs64); cudaFree(d.t_zrow); cudaFree(d.t_yrow); cudaFree(d.t_zrow_f);
     d = DeviceNet();
     Workspace &w = h->ws;
-    cudaFree(w.Vhi); cudaFree(w.Vlo); cudaFree(w.Shi); cudaFree(w.Slo); cudaFree(w.Rr16); cudaFree(w.Ri16);
+    cudaFree(w.Vhi); cudaFree(w.Vlo); cudaFree(w.Shi); cudaFree(w.Rr16); cudaFree(w.Ri16);
     cudaFree(w.RefHi); cudaFree(w.RefLo); cudaFree(w.dprev);
     cudaFree(w.Valt); cudaFree(w.fx_buf); cudaFree(w.delta_bits); cudaFree(w.delta64); cudaFree(w.iters); cudaFree(w.flags);
     cudaFree(w.rexp); cudaFree(w.tile_active); cudaFree(w.counters);
     if (w.counters_host) cudaFreeHost(w.counters_host);
+    if (w.tile_host) cudaFreeHost(w.tile_host);
     cudaFree(w.S_dev); cudaFree(w.V_dev); cudaFree(w.it_dev); cudaFree(w.mm_dev); cudaFree(w.tree_scratch);
     w = Workspace();
     if (h->tmaps) {
@@ -365,10 +384,12 @@ tpf_status ensure_workspace(tpf_handle *h, int64_t cols, int kind) {
         TPF_CK(cudaMalloc(&w.flags, sizeof(int) * cap));
         TPF_CK(cudaMalloc(&w.rexp, sizeof(int) * cap));
         TPF_CK(cudaMalloc(&w.tile_active, sizeof(int) * (cap / kTileN)));
+        if (w.tile_host) cudaFreeHost(w.tile_host);
+        w.tile_host = nullptr;
         if (have_mixed || want_mixed) {
-            cudaFree(w.Vhi); cudaFree(w.Vlo); cudaFree(w.Shi); cudaFree(w.Slo); cudaFree(w.Rr16); cudaFree(w.Ri16);
+            cudaFree(w.Vhi); cudaFree(w.Vlo); cudaFree(w.Shi); cudaFree(w.Rr16); cudaFree(w.Ri16);
             cudaFree(w.RefHi); cudaFree(w.RefLo);
-            w.Vhi = w.Vlo = w.Shi = w.Slo = w.RefHi = w.RefLo = nullptr; w.Rr16 = w.Ri16 = nullptr;
+            w.Vhi = w.Vlo = w.Shi = w.RefHi = w.RefLo = nullptr; w.Rr16 = w.Ri16 = nullptr;
         }
         if (have_fp64 || want_fp64) {
             cudaFree(w.Valt);
@@ -378,9 +399,11 @@ tpf_status ensure_workspace(tpf_handle *h, int64_t cols, int kind) {
     }
     w.n_pad = n_pad;
     const size_t el = (size_t)w.cap_cols * n_pad;
+    if (want_mixed && w.tile_host == nullptr)
+        TPF_CK(cudaMallocHost(&w.tile_host, sizeof(int) * (w.cap_cols / kTileN)));
     if (want_mixed && w.Vhi == nullptr) {
         if (cudaMalloc(&w.Vhi, sizeof(float2) * el) != cudaSuccess || cudaMalloc(&w.Vlo, sizeof(float2) * el) != cudaSuccess ||
-            cudaMalloc(&w.Shi, sizeof(float2) * el) != cudaSuccess || cudaMalloc(&w.Slo, sizeof(float2) * el) != cudaSuccess ||
+            cudaMalloc(&w.Shi, sizeof(float2) * el) != cudaSuccess ||
             cudaMalloc(&w.RefHi, sizeof(float2) * el) != cudaSuccess || cudaMalloc(&w.RefLo, sizeof(float2) * el) != cudaSuccess ||
             cudaMalloc(&w.Rr16, sizeof(__half) * el) != cudaSuccess || cudaMalloc(&w.Ri16, sizeof(__half) * el) != cudaSuccess) {
             cudaGetLastError();

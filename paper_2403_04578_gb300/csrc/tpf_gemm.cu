@@ -280,7 +280,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                             const float sc = col_scale[c0 + q];
                             const int64_t k = (n_tile * kTileN + c0 + q) * ep.n_pad + m;
                             const float2 *src = sc < 0.0f ? ep.Vlo : ep.Vhi;  // anchored: V_ref fixed
-                            old[q] = (sc != 0.0f && row_ok) ? src[k] : make_float2(0.0f, 0.0f);
+                            old[q] = make_float2(ep.v_flat ? 1.0f : 0.0f, 0.0f);
+                            if (!ep.v_flat && sc != 0.0f && row_ok) old[q] = src[k];
                         }
                         float mine = 0.0f;
 #pragma unroll

@@ -27,6 +27,7 @@ struct GemmEpi {
     int n, n_pad, k_exp;
     const int *flags, *rexp, *tile_active;
     float2 *Vhi, *Vlo;
+    int v_flat;  // every old V is 1 (the first sweep of a flat start: Vhi has not been written)
     unsigned *delta;
     // mode 2: z = D + bias[m] for rows m < real (z = 0 beyond); Dr[n][m] = z when Dr is set, and
     // Ab[n][m] = bf16(gelu(z)) (gelu != 0) or bf16(z) when Ab is set (16-bit words), both with

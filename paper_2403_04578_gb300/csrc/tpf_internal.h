@@ -119,8 +119,11 @@ struct DeviceNet {
     double *y64 = nullptr;   // complex [nnz]
     float4 *y2f = nullptr;   // double-float complex admittance (re_hi, im_hi, re_lo, im_lo) [nnz]
     bool radial = false;
-    int *par = nullptr, *ch_ptr = nullptr, *ch = nullptr;  // radial only
-    float2 *ypar = nullptr;  // FP32 admittance of the branch to the parent [n]
+    // Radial, single phase, n_pad <= 2048: what the mixed path's residual reads of a bus (tpf_residual.cu)
+    int4 *r_topo = nullptr;
+    int2 *r_inner = nullptr;
+    int r_n_inner = 0;
+    float4 *r_ypar = nullptr;  // double-float admittance of the branch to the parent [n]
     // Sparse formulation (radial only).  Block of t_threads threads per column; thread k owns the
     // t_bpt consecutive depth-first positions q = t_bpt k + j, stored at slot
     // s = j t_threads + k (so that a warp touches consecutive words).  Per slot: the column (-1
@@ -170,9 +173,9 @@ struct Workspace {
     int n_pad = 0;
     // mixed path
     // V = Vhi + Vlo: before a column is anchored Vhi carries V and Vlo = 0; after, Vhi is the
-    // frozen anchor V_ref and Vlo the offset from it.  S = Shi + Slo.  RefHi + RefLo hold
+    // frozen anchor V_ref and Vlo the offset from it.  Shi is fl(S).  RefHi + RefLo hold
     // rho(V_ref) in double-float.
-    float2 *Vhi = nullptr, *Vlo = nullptr, *Shi = nullptr, *Slo = nullptr;  // [cols][n_pad]
+    float2 *Vhi = nullptr, *Vlo = nullptr, *Shi = nullptr;                  // [cols][n_pad]
     float2 *RefHi = nullptr, *RefLo = nullptr;                              // [cols][n_pad]
     void *Rr16 = nullptr, *Ri16 = nullptr;                                  // fp16 [cols][n_pad]
     unsigned int *dprev = nullptr;        // float bits of the step before the last (mixed)
@@ -189,7 +192,8 @@ struct Workspace {
     int *rexp = nullptr;
     int *tile_active = nullptr;           // [cols / kTileN]
     int *counters = nullptr;              // [8] device counters
-    int *counters_host = nullptr;         // pinned mirror
+    int *counters_host = nullptr;         // pinned mirrors of two sweeps, 8 each
+    int *tile_host = nullptr;             // pinned mirror of tile_active
     // large-feeder sparse kernel: per-block slices of D, (S_hi, z) and the ZIP coefficients
     float4 *tree_scratch = nullptr;
     size_t tree_scratch_bytes = 0;

@@ -13,15 +13,15 @@
 // rho itself is O(n) per column: for a shunt-free network (Y V)_i = sum_j y_ij (V_i - V_j) over
 // the branches at bus i (V_slack = v_s).
 //
-// Per sweep:  mx_residual  (tpf_residual.cu, one block per column) decides convergence from the
-//                          last step, forms rho (FP32 far from convergence, then against a
-//                          double-float anchor), scales it by a per-column power of two and
-//                          writes the fp16 B operand;
+// Per sweep:  mx_tree_residual / mx_residual  (tpf_residual.cu, one block per column) decides
+//                          convergence from the last step, forms rho (FP32 far from convergence,
+//                          then against a double-float anchor), scales it by a per-column power of
+//                          two and writes the fp16 B operand;
 //             tc_gemm      (tpf_gemm.cu, persistent, warp-specialised) computes K rho with four
 //                          real-plane MMAs per K step (Re = Kr rr - Ki ri, Im = Kr ri + Ki rr)
 //                          over 128 x 128 tiles; its epilogue adds the update to V and folds
 //                          max |dV| per column.
-// This file holds the packing and output kernels and the host loop of a solve.
+// This file holds the host loop of a solve.
 #include <cuda_fp16.h>
 
 #include <cstdlib>
@@ -39,47 +39,6 @@ namespace tpf {
             return TPF_ECUDA;         \
         }                             \
     } while (0)
-
-namespace {
-
-// ------------------------------------------------------------------------------------------
-// Elementwise kernels
-// ------------------------------------------------------------------------------------------
-
-// Split S (and V_0) into double-float planes with padded rows; one block per column.  A warm start
-// (v0_lo == 0) keeps only fl32(V_0): its FP32 sweeps run on the high plane.
-__global__ void mx_pack(int64_t T, int n, int n_pad, const double2 *__restrict__ S, const double2 *__restrict__ V0,
-                        int v0_lo, float2 *Shi, float2 *Slo, float2 *Vhi, float2 *Vlo, int *flags, int *iters,
-                        unsigned *delta, unsigned *dprev) {
-    const int64_t t = blockIdx.x;
-    for (int i = threadIdx.x; i < n_pad; i += blockDim.x) {
-        float2 sh = make_float2(0.f, 0.f), sl = sh, vh = make_float2(1.f, 0.f), vl = make_float2(0.f, 0.f);
-        if (t < T && i < n) {
-            double2 s = S[t * n + i];
-            sh = make_float2(__double2float_rn(s.x), __double2float_rn(s.y));
-            sl = make_float2(__double2float_rn(s.x - (double)sh.x), __double2float_rn(s.y - (double)sh.y));
-            if (V0) {
-                double2 v = V0[t * n + i];
-                vh = make_float2(__double2float_rn(v.x), __double2float_rn(v.y));
-                if (v0_lo)
-                    vl = make_float2(__double2float_rn(v.x - (double)vh.x), __double2float_rn(v.y - (double)vh.y));
-            }
-        }
-        const int64_t k = t * n_pad + i;
-        Shi[k] = sh;
-        Slo[k] = sl;
-        Vhi[k] = vh;
-        Vlo[k] = vl;
-    }
-    if (threadIdx.x == 0) {
-        flags[t] = t < T ? kActive : 0;
-        iters[t] = 0;
-        delta[t] = 0u;
-        dprev[t] = 0u;
-    }
-}
-
-}  // namespace
 
 tpf_status selftest_gemm(int M, int N, int K, const void *Ar, const void *Ai, const void *Br, const void *Bi, float *Dr,
                          float *Di, cudaStream_t st, uint64_t wait_ns, int withhold_loads) {
@@ -111,6 +70,21 @@ tpf_status selftest_gemm(int M, int N, int K, const void *Ar, const void *Ai, co
     return herr ? TPF_ETIMEOUT : TPF_OK;
 }
 
+namespace {
+struct StreamEvent {
+    cudaEvent_t e = nullptr;
+    StreamEvent() {
+        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+            cudaGetLastError();
+            e = nullptr;
+        }
+    }
+    ~StreamEvent() {
+        if (e) cudaEventDestroy(e);
+    }
+};
+}  // namespace
+
 tpf_status solve_mixed(tpf_handle *h, int64_t T, const void *S, void *V, int32_t *iters, double *mismatch,
                        const tpf_opts &o, cudaStream_t st) {
     const int n = h->dev.n, n_pad = h->dev.n_pad;
@@ -128,17 +102,12 @@ tpf_status solve_mixed(tpf_handle *h, int64_t T, const void *S, void *V, int32_t
     int64_t launches = 0, gemm_cols = 0;
     KernelTimer timer(o.profile != 0, st);
     TPF_CK(cudaMemsetAsync(w.counters, 0, sizeof(int) * 8, st));
-    timer.begin(KernelTimer::kOther);
-    mx_pack<<<(unsigned)cols, 256, 0, st>>>(T, n, n_pad, (const double2 *)S,
-                                             o.start != TPF_START_FLAT ? (const double2 *)V : nullptr,
-                                             o.start == TPF_START_GIVEN, w.Shi, w.Slo,
-                                             w.Vhi, w.Vlo, w.flags, w.iters, w.delta_bits, w.dprev);
-    timer.end();
-    ++launches;
-    TPF_CK(cudaGetLastError());
 
     PrologueArgs pa{};
     pa.cols = cols;
+    pa.T = T;
+    pa.S64 = (const double2 *)S;
+    pa.V0 = o.start != TPF_START_FLAT ? (const double2 *)V : nullptr;
     pa.n = n;
     pa.n_pad = n_pad;
     pa.max_iter = o.max_iter;
@@ -152,16 +121,14 @@ tpf_status solve_mixed(tpf_handle *h, int64_t T, const void *S, void *V, int32_t
     pa.Vhi = w.Vhi;
     pa.Vlo = w.Vlo;
     pa.Shi = w.Shi;
-    pa.Slo = w.Slo;
     pa.RefHi = w.RefHi;
     pa.RefLo = w.RefLo;
     pa.dprev = w.dprev;
     pa.given = o.start == TPF_START_GIVEN;
-    pa.radial = h->dev.radial ? 1 : 0;
-    pa.par = h->dev.par;
-    pa.ch_ptr = h->dev.ch_ptr;
-    pa.ch = h->dev.ch;
-    pa.ypar = h->dev.ypar;
+    pa.topo = h->dev.r_topo;
+    pa.ypar4 = h->dev.r_ypar;
+    pa.inner = h->dev.r_inner;
+    pa.n_inner = h->dev.r_n_inner;
     pa.row_ptr = h->dev.row_ptr;
     pa.nbr = h->dev.nbr;
     pa.y = h->dev.y2f;
@@ -190,9 +157,11 @@ tpf_status solve_mixed(tpf_handle *h, int64_t T, const void *S, void *V, int32_t
 
     int sweeps = 0, precise_sweeps = 0;
     const int64_t n_tiles = cols / kTileN;
-    std::vector<int> tile_host(n_tiles);
+    int *const tile_host = w.tile_host;
+    StreamEvent seen;
+    if (!seen.e) return TPF_ECUDA;
     for (int s = 0; s <= o.max_iter; ++s) {
-        TPF_CK(cudaMemsetAsync(w.tile_active, 0, sizeof(int) * (cols / kTileN), st));
+        TPF_CK(cudaMemsetAsync(w.tile_active, 0, sizeof(int) * n_tiles, st));
         TPF_CK(cudaMemsetAsync(w.counters, 0, sizeof(int) * 2, st));  // active, precise
         pa.sweep = s;
         timer.begin(KernelTimer::kResidual);
@@ -200,22 +169,26 @@ tpf_status solve_mixed(tpf_handle *h, int64_t T, const void *S, void *V, int32_t
         timer.end();
         if (rs != TPF_OK) return rs;
         ++launches;
+        // The product is queued before the host has seen which tiles iterate (it skips the others), so that
+        // the host's round trip runs beside it.
         TPF_CK(cudaMemcpyAsync(w.counters_host, w.counters, sizeof(int) * 8, cudaMemcpyDeviceToHost, st));
-        TPF_CK(cudaMemcpyAsync(tile_host.data(), w.tile_active, sizeof(int) * n_tiles, cudaMemcpyDeviceToHost, st));
-        TPF_CK(cudaStreamSynchronize(st));
-        if (w.counters_host[kCntError]) return TPF_ETIMEOUT;
+        TPF_CK(cudaMemcpyAsync(tile_host, w.tile_active, sizeof(int) * n_tiles, cudaMemcpyDeviceToHost, st));
+        TPF_CK(cudaEventRecord(seen.e, st));
+        ep.v_flat = s == 0 && !pa.V0;
+        timer.begin(KernelTimer::kGemm);
+        rs = launch_gemm(maps, n_pad / kTileM, cols / kTileN, n_pad / kChunkK, ep, st);
+        timer.end();
+        if (rs != TPF_OK) return rs;
+        TPF_CK(cudaGetLastError());
+        TPF_CK(cudaEventSynchronize(seen.e));
+        if (w.counters_host[kCntError]) break;
         int64_t active = 0;
         for (int64_t k = 0; k < n_tiles; ++k) active += tile_host[k];
         if (active == 0) break;
         if (w.counters_host[kCntPrecise] > 0) ++precise_sweeps;
         gemm_cols += active;
-        timer.begin(KernelTimer::kGemm);
-        rs = launch_gemm(maps, n_pad / kTileM, cols / kTileN, n_pad / kChunkK, ep, st);
-        timer.end();
-        if (rs != TPF_OK) return rs;
         ++launches;
         ++sweeps;
-        TPF_CK(cudaGetLastError());
     }
     TPF_CK(cudaMemsetAsync(w.tile_active, 0, sizeof(int) * n_tiles, st));  // reused: converged per tile
     timer.begin(KernelTimer::kOther);
@@ -224,7 +197,7 @@ tpf_status solve_mixed(tpf_handle *h, int64_t T, const void *S, void *V, int32_t
     if (rs != TPF_OK) return rs;
     ++launches;
     TPF_CK(cudaMemcpyAsync(w.counters_host, w.counters, sizeof(int) * 8, cudaMemcpyDeviceToHost, st));
-    TPF_CK(cudaMemcpyAsync(tile_host.data(), w.tile_active, sizeof(int) * n_tiles, cudaMemcpyDeviceToHost, st));
+    TPF_CK(cudaMemcpyAsync(tile_host, w.tile_active, sizeof(int) * n_tiles, cudaMemcpyDeviceToHost, st));
     TPF_CK(cudaStreamSynchronize(st));
     int64_t converged = 0;
     for (int64_t k = 0; k < n_tiles; ++k) converged += tile_host[k];
