@@ -352,8 +352,8 @@ bool make_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows,
 
 }  // namespace
 
-bool make_bf16_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows) {
-    return make_map(map, base, inner, rows, true);
+bool make_bf16_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, uint32_t box_rows) {
+    return make_map(map, base, inner, rows, true, box_rows);
 }
 
 bool make_f16_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, uint32_t box_rows) {

@@ -42,8 +42,8 @@ struct GemmMaps {
     CUtensorMap ar, ai, br, bi;
 };
 
-// A [rows][inner] BF16 matrix read in (128 rows x 64 elements) boxes with the 128-byte swizzle.
-bool make_bf16_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows);
+// A [rows][inner] BF16 matrix read in (box_rows x 64 elements) boxes with the 128-byte swizzle.
+bool make_bf16_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, uint32_t box_rows = 128);
 // A [rows][inner] fp16 matrix read in (box_rows x 64 elements) boxes with the same swizzle.
 bool make_f16_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, uint32_t box_rows);
 // A [rows][inner] FP64 matrix (row stride inner * 8 bytes, a multiple of 16) read in unswizzled

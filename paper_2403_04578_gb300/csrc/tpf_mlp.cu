@@ -5,10 +5,11 @@
 // Features of a column: P_1..P_n, Q_1..Q_n of the demand buses (Re/Im of S), z-scored per feature;
 // targets: Re V_i - 1 and Im V_i, z-scored.  Layers z_l = W_l a_{l-1} + b_l, a_l = gelu(z_l)
 // (erf form), linear output, mean squared error, Adam.  Every matrix product runs on the
-// tcgen05 tensor cores in BF16 with FP32 accumulation (tpf_gemm.cu, real mode):
+// tcgen05 tensor cores in BF16 with FP32 accumulation:
 //   forward   Z_l  = A_{l-1} W_l^T          (A = W_l,     B = A_{l-1})
-//   weights   dW_l = dZ_l^T A_{l-1}         (A = dZ_l^T,  B = A_{l-1}^T; D comes out transposed)
 //   inputs    dA   = dZ_l W_l               (A = W_l^T,   B = dZ_l)
+//   weights   dW_l = dZ_l^T A_{l-1}         (A = dZ_l^T,  B = A_{l-1}^T; D comes out transposed)
+// in the training kernels of tpf_mlp_train.cu, layer by layer prediction on the persistent GEMM.
 // FP32 master weights, BF16 copies (W and W^T) for the products.  Feature dimensions are padded
 // to multiples of 128 and the batch to a multiple of 128; padded units stay exactly zero.
 #include <cuda_bf16.h>
@@ -21,6 +22,7 @@
 
 #include "tpf_gemm.h"
 #include "tpf_mlp_infer.h"
+#include "tpf_mlp_train.h"
 
 using bf16 = __nv_bfloat16;
 
@@ -33,6 +35,7 @@ struct tpf_mlp {
     int64_t step = 0;          // Adam step counter
     // device parameters, per layer
     std::vector<float *> W, b, mW, vW, mb, vb, gWT, gb;
+    float *flat = nullptr;     // [param_count] staging of the parameters
     std::vector<bf16 *> Wb, WTb;
     // normalisation (device, FP32): features and targets
     float *in_mean = nullptr, *in_std = nullptr, *out_mean = nullptr, *out_std = nullptr;
@@ -41,8 +44,6 @@ struct tpf_mlp {
     std::vector<float *> Z;          // pre-activations [B][pad_l]
     std::vector<bf16 *> A, AT;       // activations and transposes (hidden layers)
     std::vector<bf16 *> dZ, dZT;     // gradients of the pre-activations
-    float *dA = nullptr;             // [B][max pad]
-    float *target = nullptr;         // [B][pad_L]
     double *loss = nullptr;          // [1]
     int *err = nullptr;              // GEMM wait-expiry flag
     int *fallback = nullptr;         // [1] columns whose prediction failed the guard
@@ -69,19 +70,14 @@ namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float z) {
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
-}
-
 // The elementwise kernels run on a 2-D grid: x over the features (or units) of a column, y over
 // the columns b of the batch (grid-stride), so that no thread divides an index.
 //
 // Features of columns t0..t0+B-1 (rows beyond T are zero): x = (f - mean) / std, feature j < n
 // is Re S_j and feature n + j is Im S_j; features 2n .. P-1 are padding (zero).  Thread j reads
-// S_j once and writes both of its features, and zeroes padding feature 2n + j.
+// S_j once and writes both of its features, and zeroes padding feature 2n + j.  (Prediction only.)
 __global__ void k_features(const double2 *__restrict__ S, int64_t T, int64_t t0, int B, int n, int P,
-                           const float *__restrict__ mean, const float *__restrict__ sd, bf16 *X, bf16 *XT) {
+                           const float *__restrict__ mean, const float *__restrict__ sd, bf16 *X) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const bool feat = j < n, pad = j < P - 2 * n;
     if (!feat && !pad) return;
@@ -100,131 +96,8 @@ __global__ void k_features(const double2 *__restrict__ S, int64_t T, int64_t t0,
             const bf16 vr = __float2bfloat16_rn(xr), vi = __float2bfloat16_rn(xi);
             X[(int64_t)b * P + j] = vr;
             X[(int64_t)b * P + n + j] = vi;
-            if (XT) {
-                XT[(int64_t)j * B + b] = vr;
-                XT[(int64_t)(n + j) * B + b] = vi;
-            }
         }
-        if (pad) {
-            X[(int64_t)b * P + 2 * n + j] = zero;
-            if (XT) XT[(int64_t)(2 * n + j) * B + b] = zero;
-        }
-    }
-}
-
-// Normalised targets: (Re V - 1, Im V).
-__global__ void k_targets(const double2 *__restrict__ V, int64_t T, int64_t t0, int B, int n, int P,
-                          const float *__restrict__ mean, const float *__restrict__ sd, float *Y) {
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)B * P) return;
-    const int b = (int)(idx / P), j = (int)(idx % P);
-    const int64_t t = t0 + b;
-    float y = 0.0f;
-    if (t < T && j < 2 * n) {
-        const double2 v = V[t * n + (j < n ? j : j - n)];
-        const float f = j < n ? (float)(v.x - 1.0) : (float)v.y;
-        y = sd[j] > 0.0f ? (f - mean[j]) / sd[j] : 0.0f;
-    }
-    Y[idx] = y;
-}
-
-// z += b; a = gelu(z) (hidden) or z (output); padded units forced to zero.  AT (the transposed
-// activations, for the weight gradients) may be null.
-__global__ void k_act_fwd(float *Z, const float *__restrict__ bias, int B, int P, int real, int hidden, bf16 *A,
-                          bf16 *AT) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= P) return;
-    const float bo = o < real ? bias[o] : 0.0f;
-    for (int b = blockIdx.y; b < B; b += gridDim.y) {
-        const int64_t idx = (int64_t)b * P + o;
-        const float z = o < real ? Z[idx] + bo : 0.0f;
-        Z[idx] = z;
-        if (hidden) {
-            const bf16 a = __float2bfloat16_rn(o < real ? gelu(z) : 0.0f);
-            A[idx] = a;
-            if (AT) AT[(int64_t)o * B + b] = a;
-        }
-    }
-}
-
-// dL/dy of the mean squared error over B x real outputs, and the loss.
-__global__ void k_loss_grad(const float *__restrict__ Y, const float *__restrict__ T, int B, int P, int real,
-                            bf16 *dZ, bf16 *dZT, double *loss) {
-    __shared__ float red[kThreads / 32];
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    float sq = 0.0f;
-    if (idx < (int64_t)B * P) {
-        const int b = (int)(idx / P), o = (int)(idx % P);
-        float g = 0.0f;
-        if (o < real) {
-            const float d = Y[idx] - T[idx];
-            sq = d * d;
-            g = 2.0f * d / ((float)B * (float)real);
-        }
-        const bf16 v = __float2bfloat16_rn(g);
-        dZ[idx] = v;
-        dZT[(int64_t)o * B + b] = v;
-    }
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float s = 0.0f;
-        for (int w = 0; w < kThreads / 32; ++w) s += red[w];
-        atomicAdd(loss, (double)s / ((double)B * (double)real));
-    }
-}
-
-// dz = da * gelu'(z) for a hidden layer.
-__global__ void k_act_bwd(const float *__restrict__ dA, const float *__restrict__ Z, int B, int P, int real,
-                          bf16 *dZ, bf16 *dZT) {
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)B * P) return;
-    const int b = (int)(idx / P), o = (int)(idx % P);
-    const float g = o < real ? dA[idx] * gelu_grad(Z[idx]) : 0.0f;
-    const bf16 v = __float2bfloat16_rn(g);
-    dZ[idx] = v;
-    dZT[(int64_t)o * B + b] = v;
-}
-
-// db[o] = sum_b dZ[b][o] (one warp per output unit, rows of dZ^T are contiguous).
-__global__ void k_bias_grad(const bf16 *__restrict__ dZT, int B, int P, float *db) {
-    const int o = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (o >= P) return;
-    float s = 0.0f;
-    for (int b = lane; b < B; b += 32) s += __bfloat162float(dZT[(int64_t)o * B + b]);
-    for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
-    if (lane == 0) db[o] = s;
-}
-
-// Adam on W (gradient given transposed, gWT[k][o]) and b; then the BF16 copies W and W^T.
-__global__ void k_adam(float *W, const float *__restrict__ gWT, float *m, float *v, float *b, const float *__restrict__ gb,
-                       float *mb, float *vb, bf16 *Wb, bf16 *WTb, int Pout, int Pin, int real_out, int real_in, float lr,
-                       float b1, float b2, float eps, float c1, float c2, int update) {
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx < (int64_t)Pout * Pin) {
-        const int o = (int)(idx / Pin), k = (int)(idx % Pin);
-        float w = W[idx];
-        if (update && o < real_out && k < real_in) {
-            const float g = gWT[(int64_t)k * Pout + o];
-            const float mm = b1 * m[idx] + (1.0f - b1) * g;
-            const float vv = b2 * v[idx] + (1.0f - b2) * g * g;
-            m[idx] = mm;
-            v[idx] = vv;
-            w -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
-            W[idx] = w;
-        }
-        const bf16 wb = __float2bfloat16_rn(w);
-        Wb[idx] = wb;
-        WTb[(int64_t)k * Pout + o] = wb;
-    }
-    if (update && idx < real_out) {
-        const float g = gb[idx];
-        const float mm = b1 * mb[idx] + (1.0f - b1) * g;
-        const float vv = b2 * vb[idx] + (1.0f - b2) * g * g;
-        mb[idx] = mm;
-        vb[idx] = vv;
-        b[idx] -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+        if (pad) X[(int64_t)b * P + 2 * n + j] = zero;
     }
 }
 
@@ -336,21 +209,8 @@ __global__ void k_infer_weights(const float *__restrict__ W0, const float *__res
 
 unsigned blocks(int64_t work) { return (unsigned)((work + kThreads - 1) / kThreads); }
 
-// D[N][M] (FP32) = sum_k A[M][K] B[N][K] on the tensor cores, BF16 operands.
-tpf_status gemm_bf16(const void *A, int M, int K, const void *B, int N, float *D, int *err, cudaStream_t st) {
-    GemmMaps maps;
-    if (!make_gemm_maps(&maps, A, nullptr, M, K, B, nullptr, N, true)) return TPF_ECUDA;
-    GemmEpi ep{};
-    ep.mode = 0;
-    ep.cplx = 0;
-    ep.bf16 = 1;
-    ep.err = err;
-    ep.Dr = D;
-    ep.ldD = M;
-    return launch_gemm(maps, M / kTileM, N / kTileN, K / kChunkK, ep, st);
-}
-
-// The same product with the layer's bias and activation in the epilogue: z = D + bias for the
+// D[N][M] = sum_k A[M][K] B[N][K] on the tensor cores, BF16 operands, with the layer's bias and activation
+// in the epilogue: z = D + bias for the
 // first `real` rows; Z (FP32, may be null) receives z, Ab (may be null) bf16(gelu(z)) or bf16(z).
 tpf_status gemm_bf16_layer(const void *A, int M, int K, const void *B, int N, const float *bias, int real, bool gelu,
                            float *Z, bf16 *Ab, int *err, cudaStream_t st) {
@@ -378,7 +238,7 @@ void free_mlp(tpf_mlp *h) {
     F(h->W); F(h->b); F(h->mW); F(h->vW); F(h->mb); F(h->vb); F(h->gWT); F(h->gb); F(h->Wb); F(h->WTb);
     F(h->Z); F(h->A); F(h->AT); F(h->dZ); F(h->dZT);
     cudaFree(h->in_mean); cudaFree(h->in_std); cudaFree(h->out_mean); cudaFree(h->out_std);
-    cudaFree(h->X0); cudaFree(h->X0T); cudaFree(h->dA); cudaFree(h->target); cudaFree(h->loss); cudaFree(h->err);
+    cudaFree(h->X0); cudaFree(h->X0T); cudaFree(h->flat); cudaFree(h->loss); cudaFree(h->err);
     cudaFree(h->fallback);
     cudaFree(h->Wi0); cudaFree(h->WiL); cudaFree(h->bi_out); cudaFree(h->om_i); cudaFree(h->os_i);
     cudaFree(h->xn_i); cudaFree(h->V0c);
@@ -396,80 +256,107 @@ bool dalloc(T **p, size_t count) {
     return true;
 }
 
+// Adam's arguments; a step's settings are added by the caller.
+AdamArgs adam_args(const tpf_mlp *h) {
+    AdamArgs g{};
+    g.L = h->L;
+    for (int l = 0; l < h->L; ++l)
+        g.l[l] = AdamLayer{h->W[l], h->mW[l], h->vW[l], h->b[l], h->mb[l], h->vb[l], h->gWT[l], h->gb[l],
+                           h->Wb[l], h->WTb[l], h->pad[l + 1], h->pad[l], h->dim[l + 1], h->dim[l], 0};
+    return g;
+}
+
 // Rewrite the BF16 copies of every layer from the FP32 masters (no update).
 tpf_status publish(tpf_mlp *h, cudaStream_t st) {
     h->infer_fresh = false;
-    for (int l = 0; l < h->L; ++l) {
-        const int Po = h->pad[l + 1], Pi = h->pad[l];
-        k_adam<<<blocks((int64_t)Po * Pi), kThreads, 0, st>>>(h->W[l], h->gWT[l], h->mW[l], h->vW[l], h->b[l], h->gb[l],
-                                                              h->mb[l], h->vb[l], h->Wb[l], h->WTb[l], Po, Pi,
-                                                              h->dim[l + 1], h->dim[l], 0.f, 0.f, 0.f, 0.f, 1.f, 1.f, 0);
-    }
-    MLP_CK(cudaGetLastError());
-    return TPF_OK;
+    AdamArgs g = adam_args(h);
+    return launch_adam(g, st);
 }
 
 // 2-D grid of the elementwise kernels for B columns of P features or units.
 dim3 grid2(int P, int B) { return dim3((unsigned)((P + kThreads - 1) / kThreads), (unsigned)std::min(B, 4096)); }
 
-// Forward pass of B columns whose features are in X0; leaves Z[L-1] = normalised prediction.
-// Training also keeps every layer's Z and writes the transposed activations that the weight
-// gradients read (a pass of its own); inference takes bias and GELU in the product's epilogue.
-tpf_status forward(tpf_mlp *h, int B, cudaStream_t st, bool train) {
+// Prediction of B columns whose features are in X0, layer by layer: Z[L-1] = normalised prediction.
+tpf_status forward(tpf_mlp *h, int B, cudaStream_t st) {
     const bf16 *in = h->X0;
     for (int l = 0; l < h->L; ++l) {
         const int Po = h->pad[l + 1], Pi = h->pad[l];
         const bool hidden = l < h->L - 1;
-        if (!train) {
-            tpf_status rs = gemm_bf16_layer(h->Wb[l], Po, Pi, in, B, h->b[l], h->dim[l + 1], hidden,
-                                            hidden ? nullptr : h->Z[l], hidden ? h->A[l] : nullptr, h->err, st);
-            if (rs != TPF_OK) return rs;
-            in = hidden ? h->A[l] : nullptr;
-            continue;
-        }
-        tpf_status rs = gemm_bf16(h->Wb[l], Po, Pi, in, B, h->Z[l], h->err, st);
+        tpf_status rs = gemm_bf16_layer(h->Wb[l], Po, Pi, in, B, h->b[l], h->dim[l + 1], hidden,
+                                        hidden ? nullptr : h->Z[l], hidden ? h->A[l] : nullptr, h->err, st);
         if (rs != TPF_OK) return rs;
-        k_act_fwd<<<grid2(Po, B), kThreads, 0, st>>>(h->Z[l], h->b[l], B, Po, h->dim[l + 1], hidden,
-                                                     hidden ? h->A[l] : nullptr,
-                                                     hidden && train ? h->AT[l] : nullptr);
-        MLP_CK(cudaGetLastError());
         in = hidden ? h->A[l] : nullptr;
     }
     return TPF_OK;
 }
 
-// Backward pass after forward() with targets in h->target: fills gWT and gb of every layer.
-tpf_status backward(tpf_mlp *h, int B, cudaStream_t st) {
+// Forward and backward pass of B columns: gradients of every layer in gWT and gb, the loss.
+tpf_status gradients(tpf_mlp *h, int B, const void *S, const void *V, cudaStream_t st) {
     const int L = h->L;
-    MLP_CK(cudaMemsetAsync(h->loss, 0, sizeof(double), st));
-    k_loss_grad<<<blocks((int64_t)B * h->pad[L]), kThreads, 0, st>>>(h->Z[L - 1], h->target, B, h->pad[L], h->dim[L],
-                                                                      h->dZ[L - 1], h->dZT[L - 1], h->loss);
-    MLP_CK(cudaGetLastError());
-    for (int l = L - 1; l >= 0; --l) {
+    tpf_status rs = launch_train_features((const double2 *)S, B, h->n, h->pad[0], h->in_mean, h->in_std, h->X0, h->X0T,
+                                          h->err, h->loss, st);
+    if (rs != TPF_OK) return rs;
+    LayerArgs g{};
+    g.B = B;
+    g.V = (const double2 *)V;
+    g.n = h->n;
+    g.mean = h->out_mean;
+    g.sd = h->out_std;
+    g.loss = h->loss;
+    g.err = h->err;
+    for (int l = 0; l < L; ++l) {
+        const bool hidden = l < L - 1;
         const int Po = h->pad[l + 1], Pi = h->pad[l];
-        const bf16 *inT = l > 0 ? h->AT[l - 1] : h->X0T;
-        tpf_status rs = gemm_bf16(h->dZT[l], Po, B, inT, Pi, h->gWT[l], h->err, st);  // dW^T [Pi][Po]
+        if (!make_bf16_map(&g.a, h->Wb[l], Pi, Po) ||
+            !make_bf16_map(&g.b, l ? h->A[l - 1] : h->X0, Pi, B, kTrainN))
+            return TPF_ECUDA;
+        g.chunks = Pi / kChunkK;
+        g.M = Po;
+        g.real = h->dim[l + 1];
+        g.bias = h->b[l];
+        g.Z = h->Z[l];
+        g.o = hidden ? h->A[l] : h->dZ[l];
+        g.oT = hidden ? h->AT[l] : h->dZT[l];
+        rs = launch_layer(hidden ? kHidden : kOutput, g, st);
         if (rs != TPF_OK) return rs;
-        k_bias_grad<<<(Po * 32 + kThreads - 1) / kThreads, kThreads, 0, st>>>(h->dZT[l], B, Po, h->gb[l]);
-        MLP_CK(cudaGetLastError());
-        if (l > 0) {
-            rs = gemm_bf16(h->WTb[l], Pi, Po, h->dZ[l], B, h->dA, h->err, st);  // dA [B][Pi]
-            if (rs != TPF_OK) return rs;
-            k_act_bwd<<<blocks((int64_t)B * Pi), kThreads, 0, st>>>(h->dA, h->Z[l - 1], B, Pi, h->dim[l], h->dZ[l - 1],
-                                                                    h->dZT[l - 1]);
-            MLP_CK(cudaGetLastError());
+    }
+    for (int l = L - 1; l > 0; --l) {
+        const int Po = h->pad[l + 1], Pi = h->pad[l];
+        if (!make_bf16_map(&g.a, h->WTb[l], Po, Pi) || !make_bf16_map(&g.b, h->dZ[l], Po, B, kTrainN)) return TPF_ECUDA;
+        g.chunks = Po / kChunkK;
+        g.M = Pi;
+        g.real = h->dim[l];
+        g.Z = h->Z[l - 1];
+        g.o = h->dZ[l - 1];
+        g.oT = h->dZT[l - 1];
+        rs = launch_layer(kBackward, g, st);
+        if (rs != TPF_OK) return rs;
+    }
+    WgradArgs w{};
+    w.chunks = B / kChunkK;
+    w.err = h->err;
+    for (int l0 = 0; l0 < L; l0 += kWgradMax) {
+        w.layers = std::min(kWgradMax, L - l0);
+        for (int k = 0; k < w.layers; ++k) {
+            const int l = l0 + k, Po = h->pad[l + 1], Pi = h->pad[l];
+            if (!make_bf16_map(&w.a[k], h->dZT[l], B, Po) || !make_bf16_map(&w.b[k], l ? h->AT[l - 1] : h->X0T, B, Pi, kTrainN))
+                return TPF_ECUDA;
+            w.m_tiles[k] = Po / kTileM;
+            w.first[k + 1] = w.first[k] + Po / kTileM * (Pi / kTrainN);
+            w.D[k] = h->gWT[l];
+            w.ld[k] = Po;
+            w.zT[k] = h->dZT[l];
+            w.gb[k] = h->gb[l];
         }
+        rs = launch_wgrad(w, st);
+        if (rs != TPF_OK) return rs;
     }
     return TPF_OK;
 }
 
-tpf_status load_batch(tpf_mlp *h, int B, const void *S, const void *V, int64_t T, int64_t t0, bool transpose,
-                      cudaStream_t st) {
+tpf_status load_batch(tpf_mlp *h, int B, const void *S, int64_t T, int64_t t0, cudaStream_t st) {
     k_features<<<grid2(std::max(h->n, h->pad[0] - 2 * h->n), B), kThreads, 0, st>>>(
-        (const double2 *)S, T, t0, B, h->n, h->pad[0], h->in_mean, h->in_std, h->X0, transpose ? h->X0T : nullptr);
-    if (V)
-        k_targets<<<blocks((int64_t)B * h->pad[h->L]), kThreads, 0, st>>>(
-            (const double2 *)V, T, t0, B, h->n, h->pad[h->L], h->out_mean, h->out_std, h->target);
+        (const double2 *)S, T, t0, B, h->n, h->pad[0], h->in_mean, h->in_std, h->X0);
     MLP_CK(cudaGetLastError());
     return TPF_OK;
 }
@@ -588,8 +475,8 @@ tpf_status tpf_mlp_create(int n_pq, int hidden, int n_hidden_layers, int max_bat
     }
     ok = ok && dalloc(&h->in_mean, h->pad[0]) && dalloc(&h->in_std, h->pad[0]) && dalloc(&h->out_mean, h->pad[L]) &&
          dalloc(&h->out_std, h->pad[L]) && dalloc(&h->X0, (size_t)B * h->pad[0]) &&
-         dalloc(&h->X0T, (size_t)B * h->pad[0]) && dalloc(&h->dA, (size_t)B * maxpad) &&
-         dalloc(&h->target, (size_t)B * h->pad[L]) && dalloc(&h->loss, 1) && dalloc(&h->err, 1) &&
+         dalloc(&h->X0T, (size_t)B * h->pad[0]) && dalloc(&h->flat, (size_t)tpf_mlp_param_count(h)) &&
+         dalloc(&h->loss, 1) && dalloc(&h->err, 1) &&
          dalloc(&h->fallback, 1);
     if (!ok) {
         free_mlp(h);
@@ -641,49 +528,28 @@ int64_t tpf_mlp_param_count(const tpf_mlp *h) {
 }
 
 // Copy parameters between the device masters and a flat host array: for each layer W [out][in]
-// row-major, then b [out].
+// row-major, then b [out].  One kernel gathers or scatters them, one copy crosses to the host.
 static tpf_status params_io(tpf_mlp *h, float *host, bool to_host, bool grads) {
     if (!h || !host) return TPF_EINVAL;
     tpf::DeviceScope dscope(h->device);
     if (!dscope.ok || cudaDeviceSynchronize() != cudaSuccess) return TPF_ECUDA;
-    size_t off = 0;
+    FlatArgs g{};
+    g.L = h->L;
+    g.flat = h->flat;
+    g.mode = to_host ? (grads ? 2 : 0) : 1;
     for (int l = 0; l < h->L; ++l) {
-        const int Po = h->pad[l + 1], Pi = h->pad[l], ro = h->dim[l + 1], ri = h->dim[l];
-        std::vector<float> w((size_t)Po * Pi);
-        if (to_host) {
-            if (cudaMemcpy(w.data(), grads ? h->gWT[l] : h->W[l], sizeof(float) * w.size(), cudaMemcpyDeviceToHost) !=
-                cudaSuccess)
-                return TPF_ECUDA;
-            for (int o = 0; o < ro; ++o)
-                for (int k = 0; k < ri; ++k)
-                    host[off + (size_t)o * ri + k] = grads ? w[(size_t)k * Po + o] : w[(size_t)o * Pi + k];
-        } else {
-            std::fill(w.begin(), w.end(), 0.0f);
-            for (int o = 0; o < ro; ++o)
-                for (int k = 0; k < ri; ++k) w[(size_t)o * Pi + k] = host[off + (size_t)o * ri + k];
-            if (cudaMemcpy(h->W[l], w.data(), sizeof(float) * w.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-                return TPF_ECUDA;
-        }
-        off += (size_t)ro * ri;
-        std::vector<float> bb((size_t)Po, 0.0f);
-        if (to_host) {
-            if (cudaMemcpy(bb.data(), grads ? h->gb[l] : h->b[l], sizeof(float) * Po, cudaMemcpyDeviceToHost) !=
-                cudaSuccess)
-                return TPF_ECUDA;
-            std::memcpy(host + off, bb.data(), sizeof(float) * ro);
-        } else {
-            std::memcpy(bb.data(), host + off, sizeof(float) * ro);
-            if (cudaMemcpy(h->b[l], bb.data(), sizeof(float) * Po, cudaMemcpyHostToDevice) != cudaSuccess)
-                return TPF_ECUDA;
-        }
-        off += ro;
+        g.l[l] = FlatLayer{h->W[l], h->b[l], h->gWT[l], h->gb[l], h->pad[l + 1], h->pad[l], h->dim[l + 1], h->dim[l],
+                           g.total};
+        g.total += (int64_t)h->dim[l + 1] * h->dim[l] + h->dim[l + 1];
     }
-    if (!to_host) {
-        tpf_status rs = publish(h, nullptr);
-        if (rs != TPF_OK) return rs;
-        if (cudaDeviceSynchronize() != cudaSuccess) return TPF_ECUDA;
-    }
-    return TPF_OK;
+    const size_t bytes = sizeof(float) * (size_t)g.total;
+    if (!to_host && cudaMemcpy(h->flat, host, bytes, cudaMemcpyHostToDevice) != cudaSuccess) return TPF_ECUDA;
+    tpf_status rs = launch_flat(g, nullptr);
+    if (rs != TPF_OK) return rs;
+    if (to_host) return cudaMemcpy(host, h->flat, bytes, cudaMemcpyDeviceToHost) == cudaSuccess ? TPF_OK : TPF_ECUDA;
+    rs = publish(h, nullptr);
+    if (rs != TPF_OK) return rs;
+    return cudaDeviceSynchronize() == cudaSuccess ? TPF_OK : TPF_ECUDA;
 }
 
 tpf_status tpf_mlp_get_params(tpf_mlp *h, float *host) { return params_io(h, host, true, false); }
@@ -721,10 +587,7 @@ tpf_status tpf_mlp_gradients(tpf_mlp *h, int B, const void *S_dev, const void *V
     tpf::DeviceScope dscope(h->device);
     if (!dscope.ok) return TPF_ECUDA;
     cudaStream_t st = (cudaStream_t)stream;
-    MLP_CK(cudaMemsetAsync(h->err, 0, sizeof(int), st));
-    tpf_status rs = load_batch(h, B, S_dev, V_dev, B, 0, true, st);
-    if (rs == TPF_OK) rs = forward(h, B, st, true);
-    if (rs == TPF_OK) rs = backward(h, B, st);
+    tpf_status rs = gradients(h, B, S_dev, V_dev, st);
     if (rs == TPF_OK) rs = check_err(h, st);
     if (rs != TPF_OK) return rs;
     if (loss_out) MLP_CK(cudaMemcpy(loss_out, h->loss, sizeof(double), cudaMemcpyDeviceToHost));
@@ -738,23 +601,20 @@ tpf_status tpf_mlp_train_step(tpf_mlp *h, int B, const void *S_dev, const void *
     tpf::DeviceScope dscope(h->device);
     if (!dscope.ok) return TPF_ECUDA;
     cudaStream_t st = (cudaStream_t)stream;
-    MLP_CK(cudaMemsetAsync(h->err, 0, sizeof(int), st));
-    tpf_status rs = load_batch(h, B, S_dev, V_dev, B, 0, true, st);
-    if (rs == TPF_OK) rs = forward(h, B, st, true);
-    if (rs == TPF_OK) rs = backward(h, B, st);
+    tpf_status rs = gradients(h, B, S_dev, V_dev, st);
     if (rs != TPF_OK) return rs;
     const int64_t k = ++h->step;
     h->infer_fresh = false;
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float c1 = 1.0f - (float)std::pow(0.9, (double)k), c2 = 1.0f - (float)std::pow(0.999, (double)k);
-    for (int l = 0; l < h->L; ++l) {
-        const int Po = h->pad[l + 1], Pi = h->pad[l];
-        k_adam<<<blocks((int64_t)Po * Pi), kThreads, 0, st>>>(h->W[l], h->gWT[l], h->mW[l], h->vW[l], h->b[l], h->gb[l],
-                                                              h->mb[l], h->vb[l], h->Wb[l], h->WTb[l], Po, Pi,
-                                                              h->dim[l + 1], h->dim[l], (float)lr, b1, b2, eps, c1, c2,
-                                                              1);
-    }
-    MLP_CK(cudaGetLastError());
+    AdamArgs a = adam_args(h);
+    a.update = 1;
+    a.lr = (float)lr;
+    a.b1 = 0.9f;
+    a.b2 = 0.999f;
+    a.eps = 1e-8f;
+    a.c1 = 1.0f - (float)std::pow(0.9, (double)k);
+    a.c2 = 1.0f - (float)std::pow(0.999, (double)k);
+    rs = launch_adam(a, st);
+    if (rs != TPF_OK) return rs;
     if (loss_out) {
         MLP_CK(cudaMemcpyAsync(loss_out, h->loss, sizeof(double), cudaMemcpyDeviceToHost, st));
         return check_err(h, st);
@@ -782,8 +642,8 @@ tpf_status tpf_mlp_predict(tpf_mlp *h, int64_t T, const void *S_dev, void *V0_de
         T = 0;  // done: skip the layer-by-layer path below
     }
     for (int64_t t0 = 0; t0 < T; t0 += B) {
-        tpf_status rs = load_batch(h, B, S_dev, nullptr, T, t0, false, st);
-        if (rs == TPF_OK) rs = forward(h, B, st, false);
+        tpf_status rs = load_batch(h, B, S_dev, T, t0, st);
+        if (rs == TPF_OK) rs = forward(h, B, st);
         if (rs != TPF_OK) return rs;
         k_predict_out<<<(B * 32 + kThreads - 1) / kThreads, kThreads, 0, st>>>(
             h->Z[h->L - 1], B, h->pad[h->L], h->n, T, t0, h->out_mean, h->out_std, 0.7f, 1.1f, (double2 *)V0_dev,
