@@ -8,17 +8,27 @@
 //     V_new,q  = v_s - (prefix sum at q of E),  E_q = z_q L_q - sum of z_b L_b over the b whose
 //                                                   subtree range [b, end_b) ends at q
 //
-// (the path sum of the branch drops from the slack to q).  Every operation is FP64: this is the
-// plain double-precision fixed-point iteration of the sparse form, with Algorithm 1's per-column
-// stopping rule (max_i |V_{k+1,i} - V_{k,i}| <= tol, the first iterate that meets it is returned),
-// so that it can stand beside the mixed-precision sparse path as a like-for-like FP64 reference.
+// (the path sum of the branch drops from the slack to q).  This is the plain double-precision
+// fixed-point iteration of the sparse form, with Algorithm 1's per-column stopping rule
+// (max_i |V_{k+1,i} - V_{k,i}| <= tol, the first iterate that meets it is returned), so that it can stand
+// beside the mixed-precision sparse path as a like-for-like FP64 reference.
+//
+// GB300 issues FP64 at 1/64 of its FP32 rate, and the FP64 pipe is what bounds this kernel.  Only the
+// products and the division need it: every sum runs in 64-bit fixed point, two integer instructions
+// instead of an FP64 one that takes sixteen times as long.  Currents are integers of a last place
+// 2^cur that the sum over all buses cannot overflow (per column, from its largest load), branch terms,
+// path sums and V integers of 2^-61 pu.  Integer sums are exact, so what an FP64 prefix sum loses at its
+// own magnitude is not lost; V is rounded to FP64 where it enters a product and where it is returned.
+// The block's largest step is taken in FP32 and repeated in FP64 when it lies within 1e-5 of tol.  A column
+// that leaves the range of the integers (a current beyond four times the largest load, a drop of half a pu
+// on one branch or of 1 pu in all, anything not finite) starts again in FP64 throughout.
 //
 // One block owns one column for its whole solve, with the slot layout of the mixed kernel
 // (thread k owns depth-first positions k*bpt .. k*bpt + bpt - 1, position q at slot
 // (q % bpt) * threads + q / bpt).  V and the thread's prefix values live in registers; shared
 // memory holds S, z and one prefix array per slot (P in the first half of a sweep, the branch
-// terms in ends-list order in the second), plus the range, ends-index and parent slots.  GB300
-// issues FP64 at 1/64 of its FP32 rate, so this kernel is bound by the FP64 pipe.
+// terms in ends-list order in the second), plus the range, ends-index and parent slots.
+#include <cmath>
 #include <cstdint>
 
 #include "tpf_internal.h"
@@ -33,6 +43,10 @@ constexpr int kMaxWarps64 = kTreeMaxThreads / 32;
 struct Tree64Args {
     int n, max_iter;
     double tol2;     // tol squared: a step is compared squared
+    float tol2_lo, tol2_hi;  // tol2 in units of 2^-122 less and plus 1e-5 of itself
+    int fixed;       // sums in fixed point
+    int log2n;       // n <= 2^log2n
+    longlong2 vs_fx; // slack voltage in 2^-61 pu
     double2 vs;      // slack voltage
     const int *col, *end, *par, *ecnt, *kidx;
     const double2 *z;      // [slot] branch impedance to the parent
@@ -51,6 +65,29 @@ __device__ __forceinline__ double2 dmul(double2 a, double2 b) {
     return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }
 __device__ __forceinline__ double dabs2(double2 a) { return fma(a.x, a.x, a.y * a.y); }
+// ---- fixed point ----
+constexpr int kFx = 61;              // V, branch terms and path sums: 2^-kFx pu
+__device__ __forceinline__ int order(double v) { return ((__double2hiint(v) >> 20) & 0x7ff) - 1023; }
+// round(v * 2^s) by shifts of the significand; the caller keeps |v| * 2^s below 2^62.
+__device__ __forceinline__ long long to_fx(double v, int s) {
+    const int hi = __double2hiint(v), E = (hi >> 20) & 0x7ff, sh = E - 1075 + s;
+    const unsigned long long m =
+        ((unsigned long long)((hi & 0xfffff) | (E ? 0x100000 : 0)) << 32) | (unsigned)__double2loint(v);
+    unsigned long long x;
+    if (sh >= 0)
+        x = m << (sh & 63);
+    else
+        x = sh > -55 ? ((m >> (-sh - 1)) + 1) >> 1 : 0ull;
+    return hi < 0 ? -(long long)x : (long long)x;
+}
+// x * 2^e, rounded once (the scale by the exponent field; the results are normal numbers).
+__device__ __forceinline__ double from_fx(long long x, int e) {
+    const double d = __ll2double_rn(x);
+    return __hiloint2double(x ? __double2hiint(d) + (e << 20) : 0, __double2loint(d));
+}
+__device__ __forceinline__ longlong2 ladd(longlong2 a, longlong2 b) { return make_longlong2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ longlong2 lsub(longlong2 a, longlong2 b) { return make_longlong2(a.x - b.x, a.y - b.y); }
+
 // max that returns NaN if either operand is NaN
 __device__ __forceinline__ double dmax_nan(double m, double x) { return (m != m || x <= m) ? m : x; }
 
@@ -91,6 +128,27 @@ __device__ __forceinline__ double2 block_scan64(double2 v, double2 *wt, int lane
     return dadd(before, lane ? make_double2(ex, ey) : make_double2(0.0, 0.0));
 }
 
+// The same of integers (a lane's exclusive value as its inclusive one less its own).
+__device__ __forceinline__ longlong2 block_scan_fx(longlong2 v, longlong2 *wt, int lane, int warp, int nw) {
+    longlong2 inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long ux = __shfl_up_sync(kFull, inc.x, o), uy = __shfl_up_sync(kFull, inc.y, o);
+        if (lane >= o) inc = ladd(make_longlong2(ux, uy), inc);
+    }
+    if (lane == 31) wt[warp] = inc;
+    __syncthreads();
+    longlong2 t = lane < nw ? wt[lane] : make_longlong2(0, 0);
+    for (int o = 1; o < nw; o <<= 1) {
+        const long long ux = __shfl_up_sync(kFull, t.x, o), uy = __shfl_up_sync(kFull, t.y, o);
+        if (lane >= o) t = ladd(make_longlong2(ux, uy), t);
+    }
+    const int src = warp ? warp - 1 : 0;
+    const long long px = __shfl_sync(kFull, t.x, src), py = __shfl_sync(kFull, t.y, src);
+    const longlong2 off = lsub(inc, v);
+    return warp ? ladd(make_longlong2(px, py), off) : off;
+}
+
 template <int kBPT>
 __device__ __forceinline__ int next_slot64(int s, int th) {
     return s < (kBPT - 1) * th ? s + th : s - (kBPT - 1) * th + 1;
@@ -107,15 +165,25 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
     short *const s_rng = reinterpret_cast<short *>(dsm + 3 * ns);  // slot of the subtree's last position
     short *const s_kidx = s_rng + ns;  // where the position's branch term goes in ends-list order (-1: nowhere)
     short *const s_par = s_kidx + ns;  // parent slot, -1 = the slack
+    longlong2 *const PXi = reinterpret_cast<longlong2 *>(PX);  // the same in fixed point
     __shared__ double2 wt[kMaxWarps64];
+    longlong2 *const wti = reinterpret_cast<longlong2 *>(wt);
     __shared__ double wm[kMaxWarps64];
+    __shared__ unsigned wu[kMaxWarps64];
     const int64_t t = blockIdx.x;
     const int base = tid * kBPT;
     const double2 *S = g.S + t * n;
     double2 *Vc = g.V + t * n;
 
-    double2 V[kBPT];
+    double2 V[kBPT];  // in fixed point the bits of two integers of 2^-61 pu
+#pragma unroll
+    for (int j = 0; j < kBPT; ++j) V[j] = make_double2(1.0, 0.0);  // flat start (Algorithm 1)
     int ecnt[kBPT];
+    unsigned smax = 0;  // largest high word of the thread's loads
+    auto get_v = [&V](int j) { return make_longlong2(__double_as_longlong(V[j].x), __double_as_longlong(V[j].y)); };
+    auto set_v = [&V](int j, longlong2 x) {
+        V[j] = make_double2(__longlong_as_double(x.x), __longlong_as_double(x.y));
+    };
 #pragma unroll
     for (int j = 0; j < kBPT; ++j) {
         const int q = base + j, s = j * th + tid;
@@ -132,17 +200,139 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
             rng = (e % kBPT) * th + e / kBPT;
             if (g.given) V[j] = Vc[i];
         }
+        smax = max(smax, max((unsigned)__double2hiint(sv.x) & 0x7fffffffu, (unsigned)__double2hiint(sv.y) & 0x7fffffffu));
         Ss[s] = sv;
         Zs[s] = zv;
         s_rng[s] = (short)rng;
         s_kidx[s] = (short)g.kidx[s];
         s_par[s] = (short)g.par[s];
     }
+    smax = __reduce_max_sync(kFull, smax);
+    if (lane == 0) wu[warp] = smax;
     __syncthreads();
+    for (int w = 0; w < nw; ++w) smax = max(smax, wu[w]);
+    // Currents below 2^cur_e each (four times the largest load), so sums below 2^(cur_e + log2n):
+    // a last place of 2^cur keeps them within 62 bits.
+    const int cur_e = min(max((int)(smax >> 20) - 1022, -800), 1024) + 2, cur = cur_e + g.log2n - 62;
+    bool fixed = g.fixed && cur_e < 900, over = false;
+    if (fixed) {
+#pragma unroll
+        for (int j = 0; j < kBPT; ++j) {
+            over |= order(V[j].x) >= 1 || order(V[j].y) >= 1;
+            set_v(j, make_longlong2(to_fx(V[j].x, kFx), to_fx(V[j].y, kFx)));
+        }
+    }
 
     int it = 0;
     bool conv = false;
     for (;;) {
+        if (fixed) {
+            longlong2 loc[kBPT], run = make_longlong2(0, 0);
+#pragma unroll
+            for (int j = 0; j < kBPT; ++j) {
+                const int q = base + j, s = j * th + tid;
+                if (q < n) {
+                    const longlong2 vi = get_v(j);
+                    const double2 I = demand64<kZip>(make_double2(from_fx(vi.x, -kFx), from_fx(vi.y, -kFx)), Ss[s], g, s);
+                    over |= order(I.x) >= cur_e || order(I.y) >= cur_e;
+                    run = ladd(run, make_longlong2(to_fx(I.x, -cur), to_fx(I.y, -cur)));
+                }
+                loc[j] = run;
+            }
+            longlong2 off = block_scan_fx(run, wti, lane, warp, nw);
+#pragma unroll
+            for (int j = 0; j < kBPT; ++j) {
+                loc[j] = ladd(off, loc[j]);
+                PXi[j * th + tid] = loc[j];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int j = kBPT - 1; j >= 0; --j) {
+                const int q = base + j, s = j * th + tid;
+                longlong2 x = make_longlong2(0, 0);
+                if (q < n) {
+                    const int ls = s_rng[s];
+                    longlong2 L = ls == s ? loc[j] : PXi[ls];
+                    if (j) L = lsub(L, loc[j - 1]);
+                    else if (q > 0) L = lsub(L, PXi[(kBPT - 1) * th + tid - 1]);
+                    const double2 xd = dmul(Zs[s], make_double2(from_fx(L.x, cur), from_fx(L.y, cur)));
+                    over |= order(xd.x) >= -1 || order(xd.y) >= -1;
+                    x = make_longlong2(to_fx(xd.x, kFx), to_fx(xd.y, kFx));
+                }
+                loc[j] = x;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < kBPT; ++j) {
+                const int k = s_kidx[j * th + tid];
+                if (k >= 0) PXi[k] = loc[j];
+            }
+            __syncthreads();
+            run = make_longlong2(0, 0);
+#pragma unroll
+            for (int j = 0; j < kBPT; ++j) {
+                const int st = ecnt[j] & 0xffff, cnt = (int)(((unsigned)ecnt[j] >> 16) & 0x3fffu);
+                longlong2 e = loc[j];
+                for (int k = 0; k < cnt; ++k) e = lsub(e, PXi[st + k]);
+                run = ladd(run, e);
+                loc[j] = run;
+            }
+            off = block_scan_fx(run, wti, lane, warp, nw);
+            float m = 0.0f;
+#pragma unroll
+            for (int j = 0; j < kBPT; ++j) {
+                const int q = base + j;
+                if (q < n) {
+                    const longlong2 drop = ladd(off, loc[j]), vn = lsub(g.vs_fx, drop);
+                    const longlong2 d = lsub(vn, get_v(j));
+                    // |drop| < 1, |V_k+1| < 3, |V_k| < 3: a difference that wraps is still above 3.  (Where a
+                    // path sum itself wraps, at 4, one above it on its path lies between 1 and 4.)
+                    constexpr unsigned long long k1 = 1ull << kFx;
+                    over |= (unsigned long long)drop.x + k1 >= 2 * k1 || (unsigned long long)drop.y + k1 >= 2 * k1;
+                    const float dx = __ll2float_rn(d.x), dy = __ll2float_rn(d.y);
+                    m = fmaxf(m, fmaf(dx, dx, dy * dy));
+                    loc[j] = d;
+                    set_v(j, vn);
+                }
+            }
+            // Non-negative floats order like their bits; all ones stand for a column out of range.
+            unsigned mu = __reduce_max_sync(kFull, over ? ~0u : __float_as_uint(m));
+            if (lane == 0) wu[warp] = mu;
+            __syncthreads();
+            mu = wu[0];
+            for (int w = 1; w < nw; ++w) mu = max(mu, wu[w]);
+            if (mu == ~0u) {  // every thread alike: from the start again in FP64
+                fixed = false;
+                it = 0;
+#pragma unroll
+                for (int j = 0; j < kBPT; ++j) {
+                    const int q = base + j, s = j * th + tid;
+                    V[j] = q < n && g.given ? Vc[g.col[s]] : make_double2(1.0, 0.0);
+                }
+                continue;
+            }
+            ++it;
+            m = __uint_as_float(mu);
+            if (m <= g.tol2_hi) {
+                conv = m <= g.tol2_lo;
+                if (!conv) {  // too close to tol for FP32
+                    double md = 0.0;
+#pragma unroll
+                    for (int j = 0; j < kBPT; ++j)
+                        if (base + j < n) md = fmax(md, dabs2(make_double2(from_fx(loc[j].x, -kFx), from_fx(loc[j].y, -kFx))));
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) md = fmax(md, __shfl_xor_sync(kFull, md, o));
+                    if (lane == 0) wm[warp] = md;
+                    __syncthreads();
+                    md = wm[0];
+                    for (int w = 1; w < nw; ++w) md = fmax(md, wm[w]);
+                    conv = md <= g.tol2;
+                }
+                if (conv) break;
+            }
+            if (it >= g.max_iter) break;
+            continue;
+        }
         // Load currents and their inclusive prefix sums P.
         double2 loc[kBPT], run = make_double2(0.0, 0.0);
 #pragma unroll
@@ -216,6 +406,13 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
         if (it >= g.max_iter || !(m < 1e60)) break;
     }
 
+    if (fixed) {
+#pragma unroll
+        for (int j = 0; j < kBPT; ++j) {
+            const longlong2 x = get_v(j);
+            V[j] = make_double2(from_fx(x.x, -kFx), from_fx(x.y, -kFx));
+        }
+    }
     // Outputs: V, the iteration count, and the power mismatch max_i |V_i conj((Y v)_i) + S_i| at
     // the returned V (ZIP: |V_i| |(Y v)_i + i_d,i|).  On the tree (Y v)_q = -J_q + sum over the
     // children k of J_k with the branch currents J_k = y_k (V_parent(k) - V_k), y_k = 1 / z_k.
@@ -319,6 +516,11 @@ tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_
     g.max_iter = o.max_iter;
     g.tol2 = o.tol * o.tol;
     g.vs = make_double2(h->net.vs_re, h->net.vs_im);
+    g.tol2_lo = (float)(ldexp(g.tol2, 2 * kFx) * (1.0 - 1e-5));
+    g.tol2_hi = (float)(ldexp(g.tol2, 2 * kFx) * (1.0 + 1e-5));
+    g.fixed = fabs(g.vs.x) < 2.0 && fabs(g.vs.y) < 2.0 && o.tol < 1.0;
+    while ((1 << g.log2n) < d.n) ++g.log2n;
+    if (g.fixed) g.vs_fx = make_longlong2(llrint(ldexp(g.vs.x, kFx)), llrint(ldexp(g.vs.y, kFx)));
     g.col = d.t_col;
     g.end = d.t_end;
     g.par = d.t_par;
