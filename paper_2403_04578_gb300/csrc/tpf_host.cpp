@@ -415,9 +415,10 @@ namespace {
 // The host-buffer solve: columns are independent, so it runs chunk by chunk on the device
 // workspace (see the comment inside); solve(cols, S_dev, V_dev, iters_dev, mismatch_dev) solves one
 // chunk on `stream` and leaves its statistics in h->stats.  v_in: V_host holds a start to copy in.
+// wide: chunks of 16,384 columns and more.
 template <class Solve>
 tpf_status host_chunks(tpf_handle *h, int64_t T, const void *S_host, void *V_host, int32_t *iters_host,
-                       double *mismatch_host, const tpf_opts &o, void *stream, bool v_in, Solve solve) {
+                       double *mismatch_host, const tpf_opts &o, void *stream, bool v_in, bool wide, Solve solve) {
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     tpf::Workspace &w = h->ws;
     const size_t col_bytes = (size_t)h->net.n_pq * 16;
@@ -436,10 +437,20 @@ tpf_status host_chunks(tpf_handle *h, int64_t T, const void *S_host, void *V_hos
     // at once on an input stream, each chunk's solve waits only for its own copy, and its results go
     // back on an output stream while the next chunk is solved (pinned host memory overlaps; pageable
     // memory still works, with the copies serialised by the driver).
-    // The sparse solve is one short launch per chunk, so it takes finer chunks (less fill and drain
-    // around the copies); the dense solve's per-sweep host loop prefers fewer.
-    const int64_t max_chunks = o.method == TPF_METHOD_SPARSE ? 32 : 8;  // the learned start is sparse
-    const int64_t n_chunks = T >= 65536 ? std::min<int64_t>(max_chunks, T / 16384) : 1;
+    // The copies cost about three times the sparse solve, so its chunks only have to be large enough for their
+    // fill, drain and host round trip (100 us) not to count: sqrt(3 MB times all bytes), 16 MB at least and 32
+    // chunks at most.  Pinned, 20,160 columns of 999 buses (322 MB each way) take 4.86 ms in one chunk, 2.66 in
+    // chunks of 32 MB, 2.90 of 16 and 3.75 of 8; 5,000 columns 1.29 ms, 0.88 of 24, 0.90 of 16; 86,400 of 99
+    // buses 2.23, 1.39 of 32, 1.34 of 24, 1.68 of 8; 15 MB and less are one chunk (no difference).  The
+    // learned start predicts 128 columns per SM at a time and takes 16,384 columns at least; the dense
+    // solve's per-sweep host loop prefers few chunks.
+    const bool sparse = o.method == TPF_METHOD_SPARSE;
+    const double bytes = (double)T * (double)col_bytes, least = 16e6;
+    int64_t n_chunks = 1;
+    if (sparse && !wide)
+        n_chunks = std::max<int64_t>(1, std::min<int64_t>(32, (int64_t)(bytes / std::max(least, std::sqrt(3e6 * bytes)))));
+    else if (T >= 65536)
+        n_chunks = std::min<int64_t>(sparse ? 32 : 8, T / 16384);
     const int64_t chunk = tpf::round_up((T + n_chunks - 1) / n_chunks, tpf::kTileN);
     cudaStream_t sin = nullptr, sout = nullptr;
     std::vector<cudaEvent_t> ev;
@@ -846,7 +857,7 @@ tpf_status tpf_solve_host(tpf_handle *h, int64_t T, const void *S_host, void *V_
     if (!S_host || !V_host) return TPF_EINVAL;
     tpf::DeviceScope dscope(h->device);
     if (!dscope.ok) return TPF_ECUDA;
-    return host_chunks(h, T, S_host, V_host, iters_host, mismatch_host, o, stream, o.start != TPF_START_FLAT,
+    return host_chunks(h, T, S_host, V_host, iters_host, mismatch_host, o, stream, o.start != TPF_START_FLAT, false,
                        [&](int64_t cols, void *Sd, void *Vd, int32_t *itd, double *mmd) {
                            return tpf_solve(h, cols, Sd, Vd, itd, mmd, &o, stream);
                        });
@@ -869,7 +880,7 @@ tpf_status tpf_solve_learned_host(tpf_handle *hd, tpf_mlp *net, int64_t T, const
     tpf::DeviceScope dscope(hd->device);
     if (!dscope.ok) return TPF_ECUDA;
     int64_t fallback = 0;
-    st = host_chunks(hd, T, S_host, V_host, iters_host, mismatch_host, o, stream, false,
+    st = host_chunks(hd, T, S_host, V_host, iters_host, mismatch_host, o, stream, false, true,
                      [&](int64_t cols, void *Sd, void *Vd, int32_t *itd, double *mmd) {
                          int64_t fb = 0;
                          const tpf_status r = tpf_solve_learned(hd, net, cols, Sd, Vd, itd, mmd, &o, &fb, stream);
