@@ -88,6 +88,40 @@ __device__ __forceinline__ double from_fx(long long x, int e) {
 __device__ __forceinline__ longlong2 ladd(longlong2 a, longlong2 b) { return make_longlong2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ longlong2 lsub(longlong2 a, longlong2 b) { return make_longlong2(a.x - b.x, a.y - b.y); }
 
+// Demand current conj(s / v) of a constant-power bus in units of 2^cur, without the FP64 pipe: a quotient of
+// 25 bits in FP32, its remainder exactly in integers, and twice the same again for the remainder.
+//
+// With w the quotient so far, conj(s) - w conj(v) is taken modulo 2^64: v in 2^-53 pu (54 bits) times an
+// integer quotient of 26 bits would need 80, but the remainder is at most 2^5 quotient units times |v| and
+// fits.  Quotient units: 2^u = 2^(cur_e - 25), so that a current in range is below 2^25 of them; then 2^(u - 22);
+// the last quotient is rounded to the sum's last place 2^cur, 37 - log2n bits below 2^u.
+//   v: 2^-61 pu; s_mod: s in units of 2^(u - 53), modulo 2^64; s_f: s in units of 2^u.
+// Returns false for a current out of range (or not a number).
+__device__ __forceinline__ bool current_fx(longlong2 v, longlong2 s_mod, float2 s_f, int log2n, longlong2 &out) {
+    constexpr float k29 = 1.0f / 536870912.0f, k21 = 1.0f / 2097152.0f, k22 = 4194304.0f;
+    const float vx = (float)(int)(v.x >> 32) * k29, vy = (float)(int)(v.y >> 32) * k29;
+    const long long wx = (v.x + 128) >> 8, wy = (v.y + 128) >> 8;  // 2^-53 pu
+    const float inv = __fdividef(1.0f, fmaf(vx, vx, vy * vy));
+    const float ix = fmaf(s_f.x, vx, s_f.y * vy) * inv, iy = fmaf(s_f.x, vy, -s_f.y * vx) * inv;
+    const bool ok = fabsf(ix) < 33554432.0f && fabsf(iy) < 33554432.0f;
+    const int qx = __float2int_rn(ix), qy = __float2int_rn(iy);
+    using u64 = unsigned long long;  // modulo 2^64
+    auto mul = [](int q, long long w) { return (u64)(long long)q * (u64)w; };
+    // r = conj(s) - q conj(v), units of 2^(u - 53)
+    const u64 rx = (u64)s_mod.x - mul(qx, wx) - mul(qy, wy), ry = mul(qx, wy) - mul(qy, wx) - (u64)s_mod.y;
+    float fx = (float)(int)(rx >> 32) * k21 * inv, fy = (float)(int)(ry >> 32) * k21 * inv;
+    const int px = __float2int_rn(fmaf(fx, vx, -fy * vy) * k22), py = __float2int_rn(fmaf(fx, vy, fy * vx) * k22);
+    // the remainder of that, units of 2^(u - 75)
+    const u64 tx = (rx << 22) - mul(px, wx) - mul(py, wy), ty = (ry << 22) + mul(px, wy) - mul(py, wx);
+    fx = (float)(int)(tx >> 32) * k21 * inv, fy = (float)(int)(ty >> 32) * k21 * inv;
+    const int a = 37 - log2n, b = a - 22;
+    const float last = (float)(1 << b);
+    const int lx = __float2int_rn(fmaf(fx, vx, -fy * vy) * last), ly = __float2int_rn(fmaf(fx, vy, fy * vx) * last);
+    out.x = (long long)(((u64)(long long)qx << a) + ((u64)(long long)px << b) + (u64)(long long)lx);
+    out.y = (long long)(((u64)(long long)qy << a) + ((u64)(long long)py << b) + (u64)(long long)ly);
+    return ok;
+}
+
 // max that returns NaN if either operand is NaN
 __device__ __forceinline__ double dmax_nan(double m, double x) { return (m != m || x <= m) ? m : x; }
 
@@ -154,6 +188,10 @@ __device__ __forceinline__ int next_slot64(int s, int th) {
     return s < (kBPT - 1) * th ? s + th : s - (kBPT - 1) * th + 1;
 }
 
+// Currents in integers up to 2,048 buses (8 B more of shared memory a slot than 4,096 buses leave).
+template <int kBPT>
+constexpr bool kIntCurrents = kBPT < 8;
+
 template <int kBPT, bool kZip>
 __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : (kBPT == 2 ? 64 : 128)) f64_tree(const __grid_constant__ Tree64Args g) {
     extern __shared__ double2 dsm[];
@@ -162,7 +200,10 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
     double2 *const Ss = dsm;        // [ns] S of each position
     double2 *const Zs = dsm + ns;   // [ns] z of each position; branch currents J at the end
     double2 *const PX = dsm + 2 * ns;  // [ns] prefix sums P, then branch terms in ends-list order
-    short *const s_rng = reinterpret_cast<short *>(dsm + 3 * ns);  // slot of the subtree's last position
+    constexpr bool kInt = kIntCurrents<kBPT> && !kZip;
+    float2 *const Sf = reinterpret_cast<float2 *>(dsm + 3 * ns);   // [ns] FP32 loads of current_fx (kIntCurrents)
+    longlong2 *const Si = reinterpret_cast<longlong2 *>(Ss);       // its loads modulo 2^64, in place of Ss
+    short *const s_rng = reinterpret_cast<short *>(Sf + (kIntCurrents<kBPT> ? ns : 0));  // slot of the subtree's last position
     short *const s_kidx = s_rng + ns;  // where the position's branch term goes in ends-list order (-1: nowhere)
     short *const s_par = s_kidx + ns;  // parent slot, -1 = the slack
     longlong2 *const PXi = reinterpret_cast<longlong2 *>(PX);  // the same in fixed point
@@ -220,6 +261,13 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
         for (int j = 0; j < kBPT; ++j) {
             over |= order(V[j].x) >= 1 || order(V[j].y) >= 1;
             set_v(j, make_longlong2(to_fx(V[j].x, kFx), to_fx(V[j].y, kFx)));
+            if (kInt) {
+                const int s = j * th + tid, u = cur_e - 25;
+                const double2 sv = Ss[s];
+                const double scale = __hiloint2double((1023 - u) << 20, 0);
+                Sf[s] = make_float2(__double2float_rn(sv.x * scale), __double2float_rn(sv.y * scale));
+                Si[s] = make_longlong2(to_fx(sv.x, 53 - u), to_fx(sv.y, 53 - u));
+            }
         }
     }
 
@@ -233,9 +281,15 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
                 const int q = base + j, s = j * th + tid;
                 if (q < n) {
                     const longlong2 vi = get_v(j);
-                    const double2 I = demand64<kZip>(make_double2(from_fx(vi.x, -kFx), from_fx(vi.y, -kFx)), Ss[s], g, s);
-                    over |= order(I.x) >= cur_e || order(I.y) >= cur_e;
-                    run = ladd(run, make_longlong2(to_fx(I.x, -cur), to_fx(I.y, -cur)));
+                    if (kInt) {
+                        longlong2 I;
+                        over |= !current_fx(vi, Si[s], Sf[s], g.log2n, I);
+                        run = ladd(run, I);
+                    } else {
+                        const double2 I = demand64<kZip>(make_double2(from_fx(vi.x, -kFx), from_fx(vi.y, -kFx)), Ss[s], g, s);
+                        over |= order(I.x) >= cur_e || order(I.y) >= cur_e;
+                        run = ladd(run, make_longlong2(to_fx(I.x, -cur), to_fx(I.y, -cur)));
+                    }
                 }
                 loc[j] = run;
             }
@@ -308,6 +362,7 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
                 for (int j = 0; j < kBPT; ++j) {
                     const int q = base + j, s = j * th + tid;
                     V[j] = q < n && g.given ? Vc[g.col[s]] : make_double2(1.0, 0.0);
+                    if (kInt) Ss[s] = q < n ? S[g.col[s]] : make_double2(0.0, 0.0);
                 }
                 continue;
             }
@@ -409,8 +464,10 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
     if (fixed) {
 #pragma unroll
         for (int j = 0; j < kBPT; ++j) {
+            const int q = base + j, s = j * th + tid;
             const longlong2 x = get_v(j);
             V[j] = make_double2(from_fx(x.x, -kFx), from_fx(x.y, -kFx));
+            if (kInt) Ss[s] = q < n ? S[g.col[s]] : make_double2(0.0, 0.0);
         }
     }
     // Outputs: V, the iteration count, and the power mismatch max_i |V_i conj((Y v)_i) + S_i| at
@@ -494,7 +551,7 @@ cudaError_t launch64(int threads, int64_t cols, size_t smem, const Tree64Args &g
 
 size_t tree64_smem(int threads, int bpt) {
     const size_t ns = (size_t)threads * bpt;
-    return 3 * ns * sizeof(double2) + 3 * ns * sizeof(short);
+    return 3 * ns * sizeof(double2) + (bpt < 8 ? ns * sizeof(float2) : 0) + 3 * ns * sizeof(short);
 }
 
 tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t *iters, double *mismatch,
