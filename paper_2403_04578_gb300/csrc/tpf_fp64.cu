@@ -51,9 +51,9 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
     ++d.layout_gen;
     const int n = net.n_pq;
     cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_z);
-    cudaFree(d.t_zrow); cudaFree(d.t_yrow); cudaFree(d.t_kidx); cudaFree(d.t_zrow_f); cudaFree(d.t_z64);
+    cudaFree(d.t_zrow); cudaFree(d.t_yrow); cudaFree(d.t_kidx); cudaFree(d.t_zrow_f); cudaFree(d.t_z64); cudaFree(d.t_y64);
     cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
-    d.t_z64 = nullptr;
+    d.t_z64 = d.t_y64 = nullptr;
     d.t_topo = nullptr;
     d.t_cp = nullptr;
     d.t_zf = nullptr;
@@ -73,7 +73,7 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
             std::vector<int> col(ns, -1), end(ns, 0), par(ns, -1), ecnt(ns, 0), kidx(ns, -1);
             int n_ends = 0;  // entries of the ends lists laid out so far, in position order
             std::vector<float4> z(ns, make_float4(0.f, 0.f, 0.f, 0.f));
-            std::vector<double2> z64(ph == 1 ? ns : 0, make_double2(0.0, 0.0));
+            std::vector<double2> z64(ph == 1 ? ns : 0, make_double2(0.0, 0.0)), y64 = z64;
             // Polyphase: row p of the branch's impedance (double-float) and admittance per slot.
             std::vector<float4> zrow(ph > 1 ? (size_t)ns * ph : 0, make_float4(0.f, 0.f, 0.f, 0.f));
             std::vector<float2> yrow(ph > 1 ? (size_t)ns * ph : 0, make_float2(0.f, 0.f)), zrow_f = yrow;
@@ -98,6 +98,8 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
                 if (ph == 1) {
                     z[s] = dd(net.dfs_z[2 * q], net.dfs_z[2 * q + 1]);
                     z64[s] = make_double2(net.dfs_z[2 * q], net.dfs_z[2 * q + 1]);
+                    const double z2 = z64[s].x * z64[s].x + z64[s].y * z64[s].y;
+                    y64[s] = make_double2(z64[s].x / z2, -z64[s].y / z2);
                 } else {
                     for (int pp = 0; pp < ph; ++pp) {
                         const size_t k = (size_t)q * ph + pp;
@@ -149,7 +151,7 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
             } else if (!up(&d.t_col, col) || !up(&d.t_end, end) || !up(&d.t_par, par) || !up(&d.t_ecnt, ecnt) ||
                        !up(&d.t_z, z) || !up(&d.t_kidx, kidx) || !up(&d.t_topo, topo) || !up(&d.t_cp, cp) ||
                        !up(&d.t_zf, zf) ||
-                       (ph == 1 && !up(&d.t_z64, z64)) || (ph > 1 && (!up(&d.t_zrow, zrow) || !up(&d.t_yrow, yrow) || !up(&d.t_zrow_f, zrow_f)))) {
+                       (ph == 1 && (!up(&d.t_z64, z64) || !up(&d.t_y64, y64))) || (ph > 1 && (!up(&d.t_zrow, zrow) || !up(&d.t_yrow, yrow) || !up(&d.t_zrow_f, zrow_f)))) {
                 cudaGetLastError();
                 return TPF_ECUDA;
             }
@@ -336,7 +338,7 @@ void free_device(tpf_handle *h) {
     cudaFree(d.Kr16); cudaFree(d.Ki16); cudaFree(d.Kd16);
     cudaFree(d.r_topo); cudaFree(d.r_inner); cudaFree(d.r_ypar);
     cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_z);
-    cudaFree(d.t_kidx); cudaFree(d.t_z64); cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
+    cudaFree(d.t_kidx); cudaFree(d.t_z64); cudaFree(d.t_y64); cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
     cudaFree(d.zip64); cudaFree(d.t_zip_hi); cudaFree(d.t_zip_lo);
     cudaFree(d.csr_self); cudaFree(d.vs64); cudaFree(d.t_zrow); cudaFree(d.t_yrow); cudaFree(d.t_zrow_f);
     d = DeviceNet();

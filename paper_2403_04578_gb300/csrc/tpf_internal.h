@@ -141,7 +141,7 @@ struct DeviceNet {
     int4 *t_topo = nullptr;
     int *t_cp = nullptr;
     float2 *t_zf = nullptr;
-    double2 *t_z64 = nullptr;  // FP64 z per slot (single phase), for the FP64 sparse kernel
+    double2 *t_z64 = nullptr, *t_y64 = nullptr;  // FP64 z and 1 / z per slot (single phase), FP64 sparse kernel
     // ZIP load coefficients (Eq. 3), set by tpf_set_zip; null for constant power.  zip64: double
     // [3][n] in column order (FP64 path); t_zip_hi / t_zip_lo: float4 (alpha_P, alpha_I, alpha_Z, 0)
     // per slot, high and low words (sparse path).

@@ -28,6 +28,7 @@
 // (q % bpt) * threads + q / bpt).  V and the thread's prefix values live in registers; shared
 // memory holds S, z and one prefix array per slot (P in the first half of a sweep, the branch
 // terms in ends-list order in the second), plus the range, ends-index and parent slots.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -46,10 +47,12 @@ struct Tree64Args {
     float tol2_lo, tol2_hi;  // tol2 in units of 2^-122 less and plus 1e-5 of itself
     int fixed;       // sums in fixed point
     int log2n;       // n <= 2^log2n
+    int z_e;         // every component of z is below 2^z_e
     longlong2 vs_fx; // slack voltage in 2^-61 pu
     double2 vs;      // slack voltage
     const int *col, *end, *par, *ecnt, *kidx;
     const double2 *z;      // [slot] branch impedance to the parent
+    const double2 *y;      // [slot] its inverse
     const double *zip;     // [3][n] (alpha_P, alpha_I, alpha_Z) by column, or null
     const double2 *S;      // [T][n]
     double2 *V;            // [T][n]; read first as V_0 when given
@@ -120,6 +123,16 @@ __device__ __forceinline__ bool current_fx(longlong2 v, longlong2 s_mod, float2 
     out.x = (long long)(((u64)(long long)qx << a) + ((u64)(long long)px << b) + (u64)(long long)lx);
     out.y = (long long)(((u64)(long long)qy << a) + ((u64)(long long)py << b) + (u64)(long long)ly);
     return ok;
+}
+
+// z L in 2^-61 pu from 128-bit products (|z| < 2^61 and |L| < 2^62 in their units), rounded once; false for
+// half a pu and more.
+__device__ __forceinline__ bool branch_fx(longlong2 z, longlong2 L, int sh, longlong2 &out) {
+    const __int128 half = (__int128)1 << (sh - 1), lim = (__int128)1 << (kFx - 1);
+    const __int128 x = ((__int128)z.x * L.x - (__int128)z.y * L.y + half) >> sh;
+    const __int128 y = ((__int128)z.x * L.y + (__int128)z.y * L.x + half) >> sh;
+    out = make_longlong2((long long)x, (long long)y);
+    return x < lim && x >= -lim && y < lim && y >= -lim;
 }
 
 // max that returns NaN if either operand is NaN
@@ -203,6 +216,7 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
     constexpr bool kInt = kIntCurrents<kBPT> && !kZip;
     float2 *const Sf = reinterpret_cast<float2 *>(dsm + 3 * ns);   // [ns] FP32 loads of current_fx (kIntCurrents)
     longlong2 *const Si = reinterpret_cast<longlong2 *>(Ss);       // its loads modulo 2^64, in place of Ss
+    longlong2 *const Zi = reinterpret_cast<longlong2 *>(Zs);       // z in units of 2^(z_e - 61), in place of Zs
     short *const s_rng = reinterpret_cast<short *>(Sf + (kIntCurrents<kBPT> ? ns : 0));  // slot of the subtree's last position
     short *const s_kidx = s_rng + ns;  // where the position's branch term goes in ends-list order (-1: nowhere)
     short *const s_par = s_kidx + ns;  // parent slot, -1 = the slack
@@ -255,14 +269,19 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
     // Currents below 2^cur_e each (four times the largest load), so sums below 2^(cur_e + log2n):
     // a last place of 2^cur keeps them within 62 bits.
     const int cur_e = min(max((int)(smax >> 20) - 1022, -800), 1024) + 2, cur = cur_e + g.log2n - 62;
-    bool fixed = g.fixed && cur_e < 900, over = false;
+    // Branch terms z L: products in units of 2^(cur + z_e - 61) for a result in 2^-61 pu.
+    const int zsh = min(-(cur + g.z_e), 126);
+    bool fixed = g.fixed && cur_e < 900 && zsh >= 1, over = false;
     if (fixed) {
 #pragma unroll
         for (int j = 0; j < kBPT; ++j) {
             over |= order(V[j].x) >= 1 || order(V[j].y) >= 1;
             set_v(j, make_longlong2(to_fx(V[j].x, kFx), to_fx(V[j].y, kFx)));
+            const int s = j * th + tid;
+            const double2 zv = Zs[s];
+            Zi[s] = make_longlong2(to_fx(zv.x, 61 - g.z_e), to_fx(zv.y, 61 - g.z_e));
             if (kInt) {
-                const int s = j * th + tid, u = cur_e - 25;
+                const int u = cur_e - 25;
                 const double2 sv = Ss[s];
                 const double scale = __hiloint2double((1023 - u) << 20, 0);
                 Sf[s] = make_float2(__double2float_rn(sv.x * scale), __double2float_rn(sv.y * scale));
@@ -309,9 +328,7 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
                     longlong2 L = ls == s ? loc[j] : PXi[ls];
                     if (j) L = lsub(L, loc[j - 1]);
                     else if (q > 0) L = lsub(L, PXi[(kBPT - 1) * th + tid - 1]);
-                    const double2 xd = dmul(Zs[s], make_double2(from_fx(L.x, cur), from_fx(L.y, cur)));
-                    over |= order(xd.x) >= -1 || order(xd.y) >= -1;
-                    x = make_longlong2(to_fx(xd.x, kFx), to_fx(xd.y, kFx));
+                    over |= !branch_fx(Zi[s], L, zsh, x);
                 }
                 loc[j] = x;
             }
@@ -363,6 +380,7 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
                     const int q = base + j, s = j * th + tid;
                     V[j] = q < n && g.given ? Vc[g.col[s]] : make_double2(1.0, 0.0);
                     if (kInt) Ss[s] = q < n ? S[g.col[s]] : make_double2(0.0, 0.0);
+                    Zs[s] = q < n ? g.z[s] : make_double2(0.0, 0.0);
                 }
                 continue;
             }
@@ -461,64 +479,111 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
         if (it >= g.max_iter || !(m < 1e60)) break;
     }
 
+    // Outputs: V, the iteration count, and the power mismatch max_i |V_i conj((Y v)_i) + S_i| at
+    // the returned V (ZIP: |V_i| |(Y v)_i + i_d,i|).  On the tree (Y v)_q = -J_q + sum over the
+    // children k of J_k with the branch currents J_k = y_k (V_parent(k) - V_k), y_k = 1 / z_k.
+    // In fixed point the branch currents and their sums are integers of 2^cur like the load currents, and
+    // the largest mismatch is compared as a square.
+    double worst = 0.0;
     if (fixed) {
 #pragma unroll
         for (int j = 0; j < kBPT; ++j) {
             const int q = base + j, s = j * th + tid;
-            const longlong2 x = get_v(j);
-            V[j] = make_double2(from_fx(x.x, -kFx), from_fx(x.y, -kFx));
-            if (kInt) Ss[s] = q < n ? S[g.col[s]] : make_double2(0.0, 0.0);
-        }
-    }
-    // Outputs: V, the iteration count, and the power mismatch max_i |V_i conj((Y v)_i) + S_i| at
-    // the returned V (ZIP: |V_i| |(Y v)_i + i_d,i|).  On the tree (Y v)_q = -J_q + sum over the
-    // children k of J_k with the branch currents J_k = y_k (V_parent(k) - V_k), y_k = 1 / z_k.
-#pragma unroll
-    for (int j = 0; j < kBPT; ++j) {
-        const int q = base + j, s = j * th + tid;
-        if (q < n) Vc[g.col[s]] = V[j];
-        PX[s] = V[j];
-    }
-    __syncthreads();
-    if (g.mismatch_out) {
-#pragma unroll
-        for (int j = 0; j < kBPT; ++j) {
-            const int q = base + j, s = j * th + tid;
-            if (q < n) {
-                const int p = s_par[s];
-                const double2 zq = Zs[s];
-                const double inv = 1.0 / dabs2(zq);
-                const double2 y = make_double2(zq.x * inv, -zq.y * inv);
-                Zs[s] = dmul(y, dsub(p >= 0 ? PX[p] : g.vs, V[j]));  // the slot's own z is read first
-            }
+            const longlong2 v = get_v(j);
+            V[j] = make_double2(from_fx(v.x, -kFx), from_fx(v.y, -kFx));
+            if (q < n) Vc[g.col[s]] = V[j];
+            PXi[s] = make_longlong2(to_fx(V[j].x, kFx), to_fx(V[j].y, kFx));  // the returned V, rounded to FP64
         }
         __syncthreads();
-        double worst = 0.0;
+        longlong2 J[kBPT];
 #pragma unroll
         for (int j = 0; j < kBPT; ++j) {
             const int q = base + j, s = j * th + tid;
-            if (q < n) {
-                double2 acc = make_double2(-Zs[s].x, -Zs[s].y);
-                // The first child is q + 1; each next one follows the previous one's last position;
-                // the child whose subtree ends where q's ends is the last.
+            J[j] = make_longlong2(0, 0);
+            if (q < n && g.mismatch_out) {
+                const int p = s_par[s];
+                const longlong2 d = lsub(p >= 0 ? PXi[p] : g.vs_fx, PXi[s]);
+                const double2 i = dmul(__ldg(g.y + s), make_double2(from_fx(d.x, -kFx), from_fx(d.y, -kFx)));
+                J[j] = make_longlong2(to_fx(i.x, -cur), to_fx(i.y, -cur));
+            }
+        }
+        if (g.mismatch_out) {
+            __syncthreads();  // every parent has been read
+#pragma unroll
+            for (int j = 0; j < kBPT; ++j) PXi[j * th + tid] = J[j];
+            __syncthreads();
+            double worst2 = 0.0;
+#pragma unroll
+            for (int j = 0; j < kBPT; ++j) {
+                const int q = base + j, s = j * th + tid;
+                if (q >= n) continue;
+                longlong2 acc = make_longlong2(-J[j].x, -J[j].y);
                 const int lq = s_rng[s];
                 for (int ks = lq == s ? -1 : next_slot64<kBPT>(s, th); ks >= 0;) {
-                    acc = dadd(acc, Zs[ks]);
+                    acc = ladd(acc, PXi[ks]);
                     const int lc = s_rng[ks];
                     ks = lc == lq ? -1 : next_slot64<kBPT>(lc, th);
                 }
-                const double2 v = V[j], sv = Ss[s];
-                double mm;
-                if (kZip) {
-                    const double2 i_d = demand64<kZip>(v, sv, g, s);
-                    mm = sqrt(dabs2(v) * dabs2(dadd(acc, i_d)));
-                } else {
-                    // V conj(acc) + S
-                    mm = sqrt(dabs2(make_double2(v.x * acc.x + v.y * acc.y + sv.x, v.y * acc.x - v.x * acc.y + sv.y)));
+                const double2 a = make_double2(from_fx(acc.x, cur), from_fx(acc.y, cur)), v = V[j];
+                const double2 sv = kInt ? S[g.col[s]] : Ss[s];
+                double m2;
+                if (kZip)
+                    m2 = dabs2(v) * dabs2(dadd(a, demand64<kZip>(v, sv, g, s)));
+                else
+                    m2 = dabs2(make_double2(fma(v.x, a.x, fma(v.y, a.y, sv.x)), fma(v.y, a.x, fma(-v.x, a.y, sv.y))));
+                worst2 = fmax(worst2, m2);
+            }
+            worst = sqrt(worst2);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < kBPT; ++j) {
+            const int q = base + j, s = j * th + tid;
+            if (q < n) Vc[g.col[s]] = V[j];
+            PX[s] = V[j];
+        }
+        __syncthreads();
+        if (g.mismatch_out) {
+#pragma unroll
+            for (int j = 0; j < kBPT; ++j) {
+                const int q = base + j, s = j * th + tid;
+                if (q < n) {
+                    const int p = s_par[s];
+                    const double2 zq = Zs[s];
+                    const double inv = 1.0 / dabs2(zq);
+                    const double2 y = make_double2(zq.x * inv, -zq.y * inv);
+                    Zs[s] = dmul(y, dsub(p >= 0 ? PX[p] : g.vs, V[j]));  // the slot's own z is read first
                 }
-                worst = dmax_nan(worst, mm);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < kBPT; ++j) {
+                const int q = base + j, s = j * th + tid;
+                if (q < n) {
+                    double2 acc = make_double2(-Zs[s].x, -Zs[s].y);
+                    // The first child is q + 1; each next one follows the previous one's last position;
+                    // the child whose subtree ends where q's ends is the last.
+                    const int lq = s_rng[s];
+                    for (int ks = lq == s ? -1 : next_slot64<kBPT>(s, th); ks >= 0;) {
+                        acc = dadd(acc, Zs[ks]);
+                        const int lc = s_rng[ks];
+                        ks = lc == lq ? -1 : next_slot64<kBPT>(lc, th);
+                    }
+                    const double2 v = V[j], sv = Ss[s];
+                    double mm;
+                    if (kZip) {
+                        const double2 i_d = demand64<kZip>(v, sv, g, s);
+                        mm = sqrt(dabs2(v) * dabs2(dadd(acc, i_d)));
+                    } else {
+                        // V conj(acc) + S
+                        mm = sqrt(dabs2(make_double2(v.x * acc.x + v.y * acc.y + sv.x, v.y * acc.x - v.x * acc.y + sv.y)));
+                    }
+                    worst = dmax_nan(worst, mm);
+                }
             }
         }
+    }
+    if (g.mismatch_out) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) worst = dmax_nan(worst, __shfl_xor_sync(kFull, worst, o));
         if (lane == 0) wm[warp] = worst;  // (the last sweep's maxima were read before two barriers)
@@ -577,6 +642,13 @@ tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_
     g.tol2_hi = (float)(ldexp(g.tol2, 2 * kFx) * (1.0 + 1e-5));
     g.fixed = fabs(g.vs.x) < 2.0 && fabs(g.vs.y) < 2.0 && o.tol < 1.0;
     while ((1 << g.log2n) < d.n) ++g.log2n;
+    {
+        double zm = 0.0;
+        for (double c : h->net.dfs_z) zm = std::max(zm, std::fabs(c));
+        frexp(zm, &g.z_e);
+        if (!(zm < 1e30)) g.fixed = 0;
+        g.z_e = std::max(g.z_e, -60);
+    }
     if (g.fixed) g.vs_fx = make_longlong2(llrint(ldexp(g.vs.x, kFx)), llrint(ldexp(g.vs.y, kFx)));
     g.col = d.t_col;
     g.end = d.t_end;
@@ -584,6 +656,7 @@ tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_
     g.ecnt = d.t_ecnt;
     g.kidx = d.t_kidx;
     g.z = d.t_z64;
+    g.y = d.t_y64;
     g.zip = d.zip64;
     g.S = static_cast<const double2 *>(S);
     g.V = static_cast<double2 *>(V);
