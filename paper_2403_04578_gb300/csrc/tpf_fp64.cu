@@ -60,7 +60,7 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
     d.t_col = d.t_end = d.t_par = d.t_ecnt = d.t_kidx = nullptr;
     d.t_z = d.t_zrow = nullptr;
     d.t_yrow = d.t_zrow_f = nullptr;
-    d.t_threads = d.t_bpt = 0;
+    d.t_threads = d.t_bpt = d.t64_threads = d.t64_bpt = 0;
     if (net.radial) {
         // Slot-ordered depth-first arrays of the sparse formulation.
         const int th = bpt ? tree_threads(n, bpt) : 0;
@@ -70,10 +70,17 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
             const int ns = th * bpt;
             auto slot = [th, bpt](int q) { return (q % bpt) * th + q / bpt; };
             const int ph = net.phases, nb = n / ph;
-            std::vector<int> col(ns, -1), end(ns, 0), par(ns, -1), ecnt(ns, 0), kidx(ns, -1);
+            std::vector<int> col(ns, -1), end(ns, 0), par(ns, -1);
+            // The FP64 sparse kernel's own layout (its sums are exact, so its results do not depend on it).
+            const int bpt64 = bpt == kTreeBigBPT ? bpt : tree64_bpt(n), th64 = bpt64 == bpt ? th : tree_threads(n, bpt64);
+            const int ns64 = th64 * bpt64;
+            auto slot64 = [th64, bpt64](int q) { return (q % bpt64) * th64 + q / bpt64; };
+            std::vector<int> col64(ns64, -1), end64(ns64, 0), par64(ns64, -1), ecnt(ns64, 0), kidx(ns64, -1);
+            d.t64_threads = th64;
+            d.t64_bpt = bpt64;
             int n_ends = 0;  // entries of the ends lists laid out so far, in position order
             std::vector<float4> z(ns, make_float4(0.f, 0.f, 0.f, 0.f));
-            std::vector<double2> z64(ph == 1 ? ns : 0, make_double2(0.0, 0.0)), y64 = z64;
+            std::vector<double2> z64(ph == 1 ? ns64 : 0, make_double2(0.0, 0.0)), y64 = z64;
             // Polyphase: row p of the branch's impedance (double-float) and admittance per slot.
             std::vector<float4> zrow(ph > 1 ? (size_t)ns * ph : 0, make_float4(0.f, 0.f, 0.f, 0.f));
             std::vector<float2> yrow(ph > 1 ? (size_t)ns * ph : 0, make_float2(0.f, 0.f)), zrow_f = yrow;
@@ -88,18 +95,23 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
                 par[s] = pos_par[q] < 0 ? -1 : slot(pos_par[q]);
                 if (n_ends > 0xffff || cnt > 0x3fff) fits = false;
                 // start | count << 16 | phase << 30
-                ecnt[s] = n_ends | (cnt << 16) | ((q / nb) << 30);
+                const int s64 = slot64(q);
+                col64[s64] = net.dfs_col[q];
+                end64[s64] = net.dfs_end[q];
+                par64[s64] = pos_par[q] < 0 ? -1 : slot64(pos_par[q]);
+                ecnt[s64] = n_ends | (cnt << 16) | ((q / nb) << 30);
                 for (int k = net.dfs_eptr[q]; k < net.dfs_eptr[q + 1]; ++k)
-                    kidx[slot(net.dfs_ends[k])] = n_ends++;  // where its branch term is scattered
+                    kidx[slot64(net.dfs_ends[k])] = n_ends++;  // where its branch term is scattered
                 auto dd = [](double re, double im) {
                     const float rh = (float)re, ih = (float)im;
                     return make_float4(rh, ih, (float)(re - (double)rh), (float)(im - (double)ih));
                 };
                 if (ph == 1) {
                     z[s] = dd(net.dfs_z[2 * q], net.dfs_z[2 * q + 1]);
-                    z64[s] = make_double2(net.dfs_z[2 * q], net.dfs_z[2 * q + 1]);
-                    const double z2 = z64[s].x * z64[s].x + z64[s].y * z64[s].y;
-                    y64[s] = make_double2(z64[s].x / z2, -z64[s].y / z2);
+                    const double2 zq = make_double2(net.dfs_z[2 * q], net.dfs_z[2 * q + 1]);
+                    const double z2 = zq.x * zq.x + zq.y * zq.y;
+                    z64[s64] = zq;
+                    y64[s64] = make_double2(zq.x / z2, -zq.y / z2);
                 } else {
                     for (int pp = 0; pp < ph; ++pp) {
                         const size_t k = (size_t)q * ph + pp;
@@ -148,7 +160,7 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
             };
             if (!fits) {
                 d.t_threads = 0;
-            } else if (!up(&d.t_col, col) || !up(&d.t_end, end) || !up(&d.t_par, par) || !up(&d.t_ecnt, ecnt) ||
+            } else if (!up(&d.t_col, col64) || !up(&d.t_end, end64) || !up(&d.t_par, par64) || !up(&d.t_ecnt, ecnt) ||
                        !up(&d.t_z, z) || !up(&d.t_kidx, kidx) || !up(&d.t_topo, topo) || !up(&d.t_cp, cp) ||
                        !up(&d.t_zf, zf) ||
                        (ph == 1 && (!up(&d.t_z64, z64) || !up(&d.t_y64, y64))) || (ph > 1 && (!up(&d.t_zrow, zrow) || !up(&d.t_yrow, yrow) || !up(&d.t_zrow_f, zrow_f)))) {

@@ -619,12 +619,22 @@ size_t tree64_smem(int threads, int bpt) {
     return 3 * ns * sizeof(double2) + (bpt < 8 ? ns * sizeof(float2) : 0) + 3 * ns * sizeof(short);
 }
 
+// Buses per thread: two up to 512 buses (256 threads), where a thread's chain of sums and products is what a
+// column waits for; four up to 2,048, eight beyond (32 B of prefix sums and loads a slot).  In us, two against
+// four: 33 buses x 16,384 columns 196 and 389, 64 buses 228 and 434, 129 x 8,000 333 and 497, 299 buses 572 and 699,
+// 512 buses 865 and 872, 699 buses 1,487 and 1,287.
+int tree64_bpt(int n) {
+    for (int b : {2, 4, 8})
+        if ((b > 2 || n <= 512) && tree_threads(n, b)) return b;
+    return 0;
+}
+
 tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t *iters, double *mismatch,
                         const tpf_opts &o, cudaStream_t st) {
     const DeviceNet &d = h->dev;
     if (!d.radial || d.phases != 1 || d.t_threads == 0 || d.t_bpt == kTreeBigBPT || !d.t_z64) return TPF_EUNSUPPORTED;
     if (T > 0x7fffffff) return TPF_EUNSUPPORTED;  // one block per column
-    const size_t smem = tree64_smem(d.t_threads, d.t_bpt);
+    const size_t smem = tree64_smem(d.t64_threads, d.t64_bpt);
     if (smem > 227 * 1024) return TPF_EUNSUPPORTED;
     tpf_status rs = ensure_workspace(h, T, kWsState);  // counters
     if (rs != TPF_OK) return rs;
@@ -667,10 +677,10 @@ tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_
     KernelTimer timer(o.profile != 0, st);
     timer.begin(KernelTimer::kGemm);
     cudaError_t e;
-    switch (d.t_bpt) {
-        case 2: e = launch64<2>(d.t_threads, T, smem, g, st); break;
-        case 4: e = launch64<4>(d.t_threads, T, smem, g, st); break;
-        case 8: e = launch64<8>(d.t_threads, T, smem, g, st); break;
+    switch (d.t64_bpt) {
+        case 2: e = launch64<2>(d.t64_threads, T, smem, g, st); break;
+        case 4: e = launch64<4>(d.t64_threads, T, smem, g, st); break;
+        case 8: e = launch64<8>(d.t64_threads, T, smem, g, st); break;
         default: return TPF_EUNSUPPORTED;
     }
     timer.end();
