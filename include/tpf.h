@@ -52,7 +52,9 @@ typedef enum {
 
 /* Arithmetic of a solve. */
 enum {
-    TPF_PREC_FP64 = 0,  /* the plain double-precision fixed-point iteration (direct form)          */
+    TPF_PREC_FP64 = 0,  /* the plain fixed-point iteration (direct form) with every iterate to     *
+                         * double-precision rounding; its sums and the dense product run in exact *
+                         * fixed point where that is faster than the FP64 units                   */
     TPF_PREC_MIXED = 1  /* fp16 tensor-core sweeps with FP32 accumulation in residual form         *
                          * V <- V + K rho(V); V is carried as two floats and rho is evaluated    *
                          * against a double-float anchor, so results reach FP64-level accuracy  */
@@ -92,8 +94,8 @@ enum {
                             * fill-in-free tree substitution of a radial feeder, O(n) per column and  *
                             * sweep, the whole sweep loop of a column on chip.  TPF_PREC_MIXED: radial *
                             * networks of up to 6,144 demand unknowns (past 4,096 in chunks of 8,192  *
-                            * columns with device scratch).  TPF_PREC_FP64: the same substitution in  *
-                            * plain double precision, single-phase radial networks of up to 4,096    *
+                            * columns with device scratch).  TPF_PREC_FP64: the same substitution to  *
+                            * double precision, single-phase radial networks of up to 4,096    *
                             * demand buses (constant power or ZIP).  TPF_EUNSUPPORTED otherwise      */
 };
 
@@ -105,9 +107,10 @@ typedef struct {
     int64_t columns;      /* T of the last solve                                                */
     int64_t kernel_launches; /* kernels of this library launched by the last solve              */
     /* Filled only when opts.profile was set (milliseconds of device time, CUDA events):        */
-    double gemm_ms;          /* the dense sweep kernel: tensor-core GEMM (mixed) or FP64 sweep   */
-    double residual_ms;      /* mixed: the per-sweep residual / decision kernel; FP64: decision  */
-    double other_ms;         /* packing, initialisation and the output / mismatch kernel         */
+    double gemm_ms;          /* the dense sweep's product (mixed, FP64), the FP64 sparse kernel  */
+    double residual_ms;      /* mixed: the per-sweep residual / decision kernel; FP64: currents  *
+                              * and decision                                                     */
+    double other_ms;         /* initialisation and the output / mismatch kernel                  */
     int64_t gemm_launches;   /* launches of the dense sweep kernel                               */
     int64_t gemm_columns;    /* sum over those launches of the columns still iterating           */
 } tpf_stats;
@@ -392,8 +395,8 @@ tpf_status tpf_solve_learned_host(tpf_handle *hd, tpf_mlp *net, int64_t T, const
  * callers that must not allocate device memory themselves or have the library do it: runtimes
  * that hand out device memory only from their own pool (raw cudaMalloc/cudaFree would escape
  * their accounting), and latency-bound loops where cudaMalloc/cudaFree may synchronise the device
- * or block for an unbounded time.  It runs the same FP64 kernels as tpf_solve with
- * TPF_PREC_FP64 (Algorithm 1 in direct form, per-column stopping) but needs no handle: the
+ * or block for an unbounded time.  It runs the iteration of tpf_solve with TPF_PREC_FP64
+ * (Algorithm 1 in direct form, per-column stopping) in FP64 arithmetic throughout and needs no handle: the
  * caller passes K and W on the device, and the solve's scratch (the second V buffer and the
  * per-column state) lives in a fixed array compiled into libtpf.so.
  *

@@ -158,7 +158,7 @@ __device__ __forceinline__ float mismatch_of(float2 h, float2 l, float2 r) {
 // kP pairs of neighbouring buses per thread: 16-byte loads of the planes, half2 stores of the operand.
 // Shared memory, per bus: V or d (8 B), rho (8 B), and what its parent needs of it (16 B).
 //
-// Bound by shared-memory wavefronts (about 1,400 a column of 999 buses) and the barriers between its
+// Bound by shared-memory and L1 wavefronts (1,900 a column of 999 buses) and the barriers between its
 // phases; the bytes it must move take 48 us of an FP32 sweep of 16,384 such columns.  That sweep takes 167 us
 // (203 with every bus looping over its own children, 196 before, with parents, admittances and child lists as
 // five dependent loads a bus); an anchoring one, which is double-float arithmetic, 340 (420 before, over
