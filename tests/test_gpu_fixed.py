@@ -76,3 +76,18 @@ def test_columns_without_fixed_point_form():
         np.testing.assert_array_equal(np.isfinite(V[t]), np.isfinite(Vp[t]))
     for t in (11, 12):
         np.testing.assert_allclose(V[t], Vp[t], rtol=1e-12, atol=1e-13 * np.abs(Vp[t]).max())
+
+
+@pytest.mark.parametrize("scale", [0.1, 0.4, 1.9, 3.0])
+def test_currents_beyond_the_integer_quotient(scale):
+    # Voltages of 2 pu and more, or currents above four times the largest load, take FP64 divisions; loads ten
+    # times larger in a drop of up to 3 pu round to 15 times the bound of a sweep (3e-13 pu).
+    f = G.make_feeder(150, 9)
+    S = G.load_tensor(f, 70, 3)
+    r = np.random.default_rng(2)
+    V0 = np.ones(S.shape, complex)
+    V0[::2] = scale * np.exp(1j * r.uniform(-3.0, 3.0, (35, S.shape[1])))
+    for k in (1, 2):
+        V, it, _, Vp, itp = _both(f, S, tol=0.0, max_iter=k, V0=V0)
+        assert np.abs(V - Vp).max() <= 15 * BOUND
+        assert (it == itp).all()
