@@ -187,15 +187,6 @@ tpf_status upload_network(tpf_handle *h) {
     TPF_CK(cudaMalloc(&d.y64, sizeof(double) * 2 * (nnz > 0 ? nnz : 1)));
     TPF_CK(cudaMalloc(&d.y2f, sizeof(float4) * (nnz > 0 ? nnz : 1)));
     TPF_CK(cudaMemcpy(d.row_ptr, net.row_ptr.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice));
-    {
-        std::vector<int> order(n);
-        for (int i = 0; i < n; ++i) order[i] = i;
-        std::stable_sort(order.begin(), order.end(), [&net](int a, int b) {
-            return net.row_ptr[a + 1] - net.row_ptr[a] < net.row_ptr[b + 1] - net.row_ptr[b];
-        });
-        TPF_CK(cudaMalloc(&d.row_order, sizeof(int) * n));
-        TPF_CK(cudaMemcpy(d.row_order, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
-    }
     if (nnz > 0) {
         TPF_CK(cudaMemcpy(d.nbr, net.nbr.data(), sizeof(int) * nnz, cudaMemcpyHostToDevice));
         TPF_CK(cudaMemcpy(d.y64, net.y.data(), sizeof(double) * 2 * nnz, cudaMemcpyHostToDevice));
@@ -222,6 +213,26 @@ tpf_status upload_network(tpf_handle *h) {
         if (vs.empty()) vs = {net.vs_re, net.vs_im};
         TPF_CK(cudaMemcpy(d.vs64, vs.data(), sizeof(double) * 2 * net.phases, cudaMemcpyHostToDevice));
     }
+    if (net.radial) {
+        const tpf_status rs = layout_tree(h, tree_bpt(n));
+        if (rs != TPF_OK) return rs;
+    }
+    if (!net.K.empty()) return ensure_dense(h);  // meshed networks: K was built with the network
+    return TPF_OK;
+}
+
+// What only the dense paths read of a network besides K and W, built with them.
+static tpf_status upload_dense_lists(tpf_handle *h) {
+    const Network &net = h->net;
+    DeviceNet &d = h->dev;
+    const int n = d.n;
+    if (d.row_order) return TPF_OK;
+    cudaFree(d.r_topo);  // (of an upload that failed half-way)
+    cudaFree(d.r_inner);
+    cudaFree(d.r_ypar);
+    d.r_topo = nullptr;
+    d.r_inner = nullptr;
+    d.r_ypar = nullptr;
     if (net.radial && net.phases == 1 && d.n_pad <= 2048) {
         std::vector<int4> topo(n);
         std::vector<float4> yp(n);
@@ -252,11 +263,15 @@ tpf_status upload_network(tpf_handle *h) {
         TPF_CK(cudaMemcpy(d.r_topo, topo.data(), sizeof(int4) * n, cudaMemcpyHostToDevice));
         TPF_CK(cudaMemcpy(d.r_ypar, yp.data(), sizeof(float4) * n, cudaMemcpyHostToDevice));
     }
-    if (net.radial) {
-        const tpf_status rs = layout_tree(h, tree_bpt(n));
-        if (rs != TPF_OK) return rs;
+    {
+        std::vector<int> order(n);
+        for (int i = 0; i < n; ++i) order[i] = i;
+        std::stable_sort(order.begin(), order.end(), [&net](int a, int b) {
+            return net.row_ptr[a + 1] - net.row_ptr[a] < net.row_ptr[b + 1] - net.row_ptr[b];
+        });
+        TPF_CK(cudaMalloc(&d.row_order, sizeof(int) * n));
+        TPF_CK(cudaMemcpy(d.row_order, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
     }
-    if (!net.K.empty()) return ensure_dense(h);  // meshed networks: K was built with the network
     return TPF_OK;
 }
 
@@ -266,6 +281,8 @@ tpf_status ensure_dense(tpf_handle *h) {
     Network &net = h->net;
     try {
         compute_dense(net);
+        const tpf_status rs = upload_dense_lists(h);
+        if (rs != TPF_OK) return rs;
     } catch (const std::bad_alloc &) {
         return TPF_ENOMEM;
     }
