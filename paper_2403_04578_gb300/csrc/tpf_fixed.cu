@@ -4,19 +4,23 @@
 // GB300 runs FP64 at 1/64 of its FP32 rate (1.2 TFLOP/s) and fp16 on the tensor cores at 1.9
 // PFLOP/s, so the 8 n^2 FP64 operations of a column and sweep are replaced by integer arithmetic
 // (the splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012, with digits of equal
-// place instead of floating slices).  Every component of K (scaled once by the largest) and of the
-// injections I = conj(S ./ V) (scaled per column by that column's largest) becomes an integer of at
-// most 2^55, so that the largest one keeps its whole FP64 significand, written as seven balanced
-// base-256 digits d_0 .. d_6 in [-128, 128], each exact in fp16.  Then
+// place instead of floating slices).  Bus j's column of K is divided by a power of two c_j, its largest
+// component's order, and its current multiplied by it: J_j = c_j I_j is the largest voltage drop that the bus
+// causes by itself, whatever the decades between impedances (an open switch modelled as one of 1e6 pu) or
+// between loads.  Every component of K / c and of J (scaled per column of the tensor by that column's largest)
+// becomes an integer of at most 2^55, so that the largest one keeps its whole FP64 significand, written as
+// seven balanced base-256 digits d_0 .. d_6 in [-128, 128], each exact in fp16.  Then
 //
-//     K I = sum over diagonals d of 256^-d  sum_{i + j = d} K_i I_j
+//     K I = (K / c) J = sum over diagonals d of 256^-d  sum_{i + j = d} (K / c)_i J_j
 //
-// with the diagonals 0 .. 6 kept (28 digit products; what is dropped is below 2^-50 of the product of
-// the two scales for 1,000 buses, and such a product is itself one bus's share of the voltage drop).
+// with the diagonals 0 .. 6 kept (28 digit products).  In units of the column's largest J, what is dropped
+// is 2^-51 (root mean square, digits of no pattern) at 1,000 buses, 2^-42.4 at the very worst (12 n products
+// of 2^14 two places below diagonal 6, all of one sign); J is below 2^-8 pu on the feeders of inputs.py.  With
+// one scale for all of K and one for all currents, as this once was, an unloaded stub of 1e6 pu cost the other
+// buses of a 200-bus feeder 1.3e-10 pu, and one load of 1,000 pu near the source 6.2e-14.
 // A digit product's sum over 512 terms stays below 2^24, so the FP32 accumulators in TMEM hold it
 // exactly whatever the order; the accumulated integers are then added in 64-bit integer arithmetic,
-// down to a last place that the sum of all n terms cannot overflow (2^-53 of the two scales' product at
-// 256 buses).  A column's result therefore does not depend on the tile it falls in.
+// down to a last place that the sum of all n terms cannot overflow (2^-53 of the largest J at 256 buses).  A column's result therefore does not depend on the tile it falls in.
 //
 // Measured against binary128 on one sweep from random starts, the largest error is 5.5e-17 to 7e-17 pu at
 // 1 to 399 buses (half a last place of V: the only rounding left is that of the result), where the FP64
@@ -65,7 +69,7 @@ constexpr int kFxEpiWarps = 8;
 constexpr int kFxEpiThreads = 32 * kFxEpiWarps;
 constexpr int kFxThreads = 64 + kFxEpiThreads;
 constexpr uint32_t kFxAcc = 4 * kFxN;  // TMEM columns of a stage: Re, Im of the upper and the lower diagonal
-constexpr int kMinExp = -900, kMaxExp = 1000;  // binary orders of a column's largest current
+constexpr int kMinExp = -900, kMaxExp = 1000;  // binary orders of a column's largest J
 constexpr int kFxMaxN = 8192;                  // fx_slice keeps a column's currents in shared memory
 
 // Counters of the sweeps: columns left to fx_column, and the lengths of the two column lists (a sweep reads
@@ -77,9 +81,9 @@ struct FxArgs {
     const int *count;     // device: columns that iterate
     int first, cap;       // this launch takes those from `first`, at most cap (the rows of a digit plane of I)
     const int *list;      // the columns, or null: 0, 1, ...
-    double f1;            // 2^(drop - 62 + exponent of K): value of a last place for a column of order 0
+    double f1;            // 2^(drop - 62 + order of K / c): value of a last place for a column of order 0
     int drop;             // last place of the 64-bit sums, in bits above diagonal 6's
-    const int *colexp;    // per column of this launch: binary order of the largest current; kMaxExp: skip
+    const int *colexp;    // per column of this launch: binary order of the largest J; kMaxExp: skip
     const double2 *W;
     double2 *V;
     unsigned long long *delta;
@@ -111,12 +115,14 @@ __device__ __forceinline__ long long to_fixed(double v, int e) {
     return (long long)b < 0 ? -(long long)x : (long long)x;
 }
 
-// Digit planes [kDig][n_pad][n_pad] of K * 2^(kBits - exponent of K), zero padded.
-__global__ void fx_k_digits(const double2 *__restrict__ K, int n, int n_pad, double scale, __half *Kr, __half *Ki) {
+// Digit planes [kDig][n_pad][n_pad] of K * 2^(shift - order of the column), zero padded.
+__global__ void fx_k_digits(const double2 *__restrict__ K, const int *__restrict__ col_order, int n, int n_pad,
+                            int shift, __half *Kr, __half *Ki) {
     const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, plane = (int64_t)n_pad * n_pad;
     if (idx >= plane) return;
     const int i = (int)(idx / n_pad), j = (int)(idx % n_pad);
     double2 k = make_double2(0.0, 0.0);
+    const double scale = j < n ? ldexp(1.0, shift - col_order[j]) : 0.0;
     if (i < n && j < n) k = K[(size_t)i * n + j];
     __half dr[kDig], di[kDig];
     digits(__double2ll_rn(k.x * scale), dr);
@@ -160,16 +166,17 @@ __device__ __forceinline__ float scaled_f(double v, int u) {
     return E > 0 ? __int_as_float(bits) : 0.0f;
 }
 
-// Injections of one column per block and their digit planes [kDig][cap][n_pad] (re, im, -re).  The largest
-// component's order comes from the high words (an ordered integer maximum; NaN is above infinity).
+// Injections J of one column per block and their digit planes [kDig][cap][n_pad] (re, im, -re).  The largest
+// component's order comes from the high words (an ordered integer maximum; NaN is above infinity).  c_j is a
+// power of two, so J is the current of a load c_j S.
 // Constant-power currents of voltages below 2 pu come from integer remainders (current_fx), the others, ZIP loads
 // and columns out of its range from FP64 divisions, which bound the kernel: 23.7 instead of 30.2 us for 4,800
 // columns of 199 buses (the bytes of S, V and the planes take 13), 1.83 instead of 1.92 ms for a solve of 8,760.
 __global__ void __launch_bounds__(kSliceThreads)
     fx_slice(int n, int n_pad, const int *__restrict__ list, const int *count, int first,
              const double2 *__restrict__ S,
-             const double2 *__restrict__ V, const double *__restrict__ zip, __half *Dr, __half *Di, __half *Dn, int cap,
-             int *colexp, int *plain, int *counters) {
+             const double2 *__restrict__ V, const double *__restrict__ zip, const int *__restrict__ col_order,
+             __half *Dr, __half *Di, __half *Dn, int cap, int *colexp, int *plain, int *counters) {
     extern __shared__ double2 cur[];
     __shared__ unsigned s_max[3][kSliceThreads / 32];
     longlong2 *const cur_i = reinterpret_cast<longlong2 *>(cur);
@@ -192,21 +199,27 @@ __global__ void __launch_bounds__(kSliceThreads)
     bool ints = false;
     int cut = 0;
     if (!zip) {
-        // Constant power, |V| below 2 pu, currents below four times the largest load: in integers of 2^(e - 58)
+        // Constant power, |V| below 2 pu, J below four times the largest c_j S: in integers of 2^(e - 58)
         // at once (current_fx with four bits of headroom), cut to the 55 bits that the largest one needs.
-        for (int i = tid; i < n; i += kSliceThreads) m = max(m, top(S[t * n + i]));
+        // Orders of the scaled loads; zeros and denormals count as none, infinities and NaN as the largest.
+        for (int i = tid; i < n; i += kSliceThreads) {
+            const int o = (int)(top(S[t * n + i]) >> 20);
+            const int so = o == 0 ? 0 : (o == 0x7ff ? 4095 : max(o + col_order[i], 0));
+            m = max(m, (unsigned)so);
+        }
         m = block_max(m, 0);
-        e = min(max((int)(m >> 20) - 1022, -800), 1024) + 2;
+        e = min(max((int)m - 1022, -800), 1024) + 2;
         if (e < 900) {
             const int u = e - 25;
             bool over = false;
             unsigned mx = 0;
             for (int i = tid; i < n; i += kSliceThreads) {
                 const double2 s = S[t * n + i], v = V[t * n + i];
+                const int c = col_order[i];
                 over |= order(v.x) >= 1 || order(v.y) >= 1;
                 over |= !current_fx(make_longlong2(to_fx(v.x, kFx), to_fx(v.y, kFx)),
-                                    make_longlong2(to_fx(s.x, 53 - u), to_fx(s.y, 53 - u)),
-                                    make_float2(scaled_f(s.x, u), scaled_f(s.y, u)), 4, cur_i[i]);
+                                    make_longlong2(to_fx(s.x, 53 - u + c), to_fx(s.y, 53 - u + c)),
+                                    make_float2(scaled_f(s.x, u - c), scaled_f(s.y, u - c)), 4, cur_i[i]);
                 const longlong2 x = cur_i[i];
                 mx = max(mx, (unsigned)(max(llabs(x.x), llabs(x.y)) >> 32));
             }
@@ -222,8 +235,9 @@ __global__ void __launch_bounds__(kSliceThreads)
         m = 0;
         for (int i = tid; i < n; i += kSliceThreads) {
             const double2 I = demand(S[t * n + i], V[t * n + i], zip, n, i);
-            cur[i] = I;
-            m = max(m, top(I));
+            const double c = pow2d(col_order[i]);
+            cur[i] = make_double2(I.x * c, I.y * c);
+            m = max(m, top(cur[i]));
         }
         m = block_max(m, 2);
         e = (int)(m >> 20) - 1022;
@@ -644,7 +658,7 @@ tpf_status solve_fixed(tpf_handle *h, int64_t T, const void *S, void *V, const t
     DeviceNet &d = h->dev;
     const int n = d.n, n_pad = d.n_pad;
     const size_t plane_k = (size_t)n_pad * n_pad;
-    const int k_order = 14 - d.k_exp;  // every component of K is below 2^k_order
+    const int k_order = d.k_order;  // every component of K / c is below 2^k_order
     int64_t launches = 0, gemms = 0, gemm_cols = 0;
     if (!d.Kd16) {
         if (cudaMalloc(&d.Kd16, sizeof(__half) * 2 * kDig * plane_k) != cudaSuccess) {
@@ -652,8 +666,8 @@ tpf_status solve_fixed(tpf_handle *h, int64_t T, const void *S, void *V, const t
             d.Kd16 = nullptr;
             return TPF_ENOMEM;
         }
-        fx_k_digits<<<(unsigned)((plane_k + 255) / 256), 256, 0, st>>>((const double2 *)d.K64, n, n_pad,
-                                                                       ldexp(1.0, kBits - k_order), (__half *)d.Kd16,
+        fx_k_digits<<<(unsigned)((plane_k + 255) / 256), 256, 0, st>>>((const double2 *)d.K64, d.k_col_order, n, n_pad,
+                                                                       kBits - k_order, (__half *)d.Kd16,
                                                                        (__half *)d.Kd16 + kDig * plane_k);
         TPF_CK(cudaGetLastError());
         ++launches;
@@ -737,8 +751,8 @@ tpf_status solve_fixed(tpf_handle *h, int64_t T, const void *S, void *V, const t
             g.first = (int)c0;
             timer.begin(KernelTimer::kResidual);
             fx_slice<<<(unsigned)cnt, kSliceThreads, smem, st>>>(n, n_pad, list, g.count, g.first, (const double2 *)S,
-                                                                 (const double2 *)V, d.zip64, Dr, Di, Dn, (int)cap,
-                                                                 colexp, plain, w.counters);
+                                                                 (const double2 *)V, d.zip64, d.k_col_order, Dr, Di, Dn,
+                                                                 (int)cap, colexp, plain, w.counters);
             timer.end();
             const int total = g.m_tiles * ((cnt + kFxN - 1) / kFxN);
             timer.begin(KernelTimer::kGemm);

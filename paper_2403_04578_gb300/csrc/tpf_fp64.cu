@@ -275,13 +275,41 @@ static tpf_status upload_dense_lists(tpf_handle *h) {
     return TPF_OK;
 }
 
+// Binary orders of K's columns (DeviceNet), from the host's K.
+static tpf_status upload_column_orders(tpf_handle *h) {
+    const std::vector<double> &K = h->net.K;
+    DeviceNet &d = h->dev;
+    const int n = d.n;
+    if (K.size() != 2 * (size_t)n * n) return TPF_ESINGULAR;
+    std::vector<double> top(n, 0.0);
+    for (int i = 0; i < n; ++i)
+        for (int j = 0; j < n; ++j) {
+            const double *k = &K[2 * ((size_t)i * n + j)];
+            top[j] = std::max(top[j], std::max(std::fabs(k[0]), std::fabs(k[1])));
+        }
+    std::vector<int> order(n);
+    d.k_order = -2000;
+    for (int j = 0; j < n; ++j) {
+        int o = 0;
+        if (top[j] > 0.0) frexp(top[j], &o);
+        order[j] = std::min(std::max(o, -100), 100);
+        d.k_order = std::max(d.k_order, o - order[j]);
+    }
+    cudaFree(d.k_col_order);  // (of a call that failed half-way)
+    d.k_col_order = nullptr;
+    TPF_CK(cudaMalloc(&d.k_col_order, sizeof(int) * n));
+    TPF_CK(cudaMemcpy(d.k_col_order, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
+    return TPF_OK;
+}
+
 tpf_status ensure_dense(tpf_handle *h) {
     DeviceNet &d = h->dev;
     if (d.K64) return TPF_OK;
     Network &net = h->net;
     try {
         compute_dense(net);
-        const tpf_status rs = upload_dense_lists(h);
+        tpf_status rs = upload_dense_lists(h);
+        if (rs == TPF_OK) rs = upload_column_orders(h);
         if (rs != TPF_OK) return rs;
     } catch (const std::bad_alloc &) {
         return TPF_ENOMEM;
@@ -364,7 +392,7 @@ tpf_status set_zip(tpf_handle *h, const double *alpha) {
 void free_device(tpf_handle *h) {
     DeviceNet &d = h->dev;
     cudaFree(d.K64); cudaFree(d.W64); cudaFree(d.row_ptr); cudaFree(d.nbr); cudaFree(d.row_order); cudaFree(d.y64); cudaFree(d.y2f);
-    cudaFree(d.Kr16); cudaFree(d.Ki16); cudaFree(d.Kd16);
+    cudaFree(d.Kr16); cudaFree(d.Ki16); cudaFree(d.Kd16); cudaFree(d.k_col_order);
     cudaFree(d.r_topo); cudaFree(d.r_inner); cudaFree(d.r_ypar);
     cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_z);
     cudaFree(d.t_kidx); cudaFree(d.t_z64); cudaFree(d.t_y64); cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);

@@ -162,7 +162,10 @@ struct DeviceNet {
     // Mixed path: fp16 planes of K * 2^k_exp, [n_pad][n_pad], zero padded
     void *Kr16 = nullptr, *Ki16 = nullptr;
     int k_exp = 0;
-    // FP64 path on the tensor cores: fp16 digit planes of K (Re, then Im), [2][7][n_pad][n_pad]
+    // FP64 path on the tensor cores: per bus j the order of its column of K (every |K_ij| < 2^(k_order +
+    // order), k_order 0 for columns between 2^-100 and 2^100), and the fp16 digit planes of the columns so
+    // scaled (Re, then Im), [2][7][n_pad][n_pad]
+    int *k_col_order = nullptr, k_order = 0;
     void *Kd16 = nullptr;
     // Incremented whenever the sparse layout or the ZIP coefficients are replaced: a prepared
     // batch (tpf_batch) that captured the old device arrays then refuses to launch.
