@@ -169,7 +169,7 @@ __device__ __forceinline__ float scaled_f(double v, int u) {
 // Injections J of one column per block and their digit planes [kDig][cap][n_pad] (re, im, -re).  The largest
 // component's order comes from the high words (an ordered integer maximum; NaN is above infinity).  c_j is a
 // power of two, so J is the current of a load c_j S.
-// Constant-power currents of voltages below 2 pu come from integer remainders (current_fx), the others, ZIP loads
+// Constant-power currents of voltages from 0.5 to 2 pu come from integer remainders (current_fx), the others, ZIP loads
 // and columns out of its range from FP64 divisions, which bound the kernel: 23.7 instead of 30.2 us for 4,800
 // columns of 199 buses (the bytes of S, V and the planes take 13), 1.83 instead of 1.92 ms for a solve of 8,760.
 __global__ void __launch_bounds__(kSliceThreads)
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kSliceThreads)
     bool ints = false;
     int cut = 0;
     if (!zip) {
-        // Constant power, |V| below 2 pu, J below four times the largest c_j S: in integers of 2^(e - 58)
+        // Constant power, |V| from 0.5 to 2 pu, J below four times the largest c_j S: in integers of 2^(e - 58)
         // at once (current_fx with four bits of headroom), cut to the 55 bits that the largest one needs.
         // Orders of the scaled loads; zeros and denormals count as none, infinities and NaN as the largest.
         for (int i = tid; i < n; i += kSliceThreads) {

@@ -20,22 +20,34 @@ __device__ __forceinline__ long long to_fx(double v, int s) {
     return hi < 0 ? -(long long)x : (long long)x;
 }
 
+// |v|^2 in FP32 of v in 2^-61 pu, from the high words.
+__device__ __forceinline__ float abs2_fx(longlong2 v) {
+    constexpr float k29 = 1.0f / 536870912.0f;
+    const float x = (float)(int)(v.x >> 32) * k29, y = (float)(int)(v.y >> 32) * k29;
+    return fmaf(x, x, y * y);
+}
+// Below half a pu the integers' last places, 2^-61 pu here and 2^-53 in current_fx, are no longer far enough
+// below v: such a voltage's current is an FP64 division of an FP64 voltage.  (The quotients of current_fx lose
+// bits in proportion to 1 / |v|, and wrap below 1e-4 pu; converged voltages of a feeder are above 0.5 pu.)
+constexpr float kLowV2 = 0.25f;
+
 // Demand current conj(s / v) of a constant-power bus in units of 2^cur, without the FP64 pipe: a quotient of
 // 25 bits in FP32, its remainder exactly in integers, and twice the same again for the remainder.
 //
 // With w the quotient so far, conj(s) - w conj(v) is taken modulo 2^64: v in 2^-53 pu (54 bits) times an
 // integer quotient of 26 bits would need 80, but the remainder is at most 2^5 quotient units times |v| and
-// fits.  Quotient units: 2^u = 2^(cur_e - 25), so that a current in range is below 2^25 of them; then 2^(u - 22);
+// fits (|v| at least half a pu: the FP32 quotient's own error is 2^-29 / |v|, five bits of it in quotient units).
+// Quotient units: 2^u = 2^(cur_e - 25), so that a current in range is below 2^25 of them; then 2^(u - 22);
 // the last quotient is rounded to the sum's last place 2^cur, 37 - log2n bits below 2^u.
 //   v: 2^-61 pu; s_mod: s in units of 2^(u - 53), modulo 2^64; s_f: s in units of 2^u.
-// Returns false for a current out of range (or not a number).
+// Returns false for a current out of range (or not a number) and for |v| below half a pu.
 __device__ __forceinline__ bool current_fx(longlong2 v, longlong2 s_mod, float2 s_f, int log2n, longlong2 &out) {
     constexpr float k29 = 1.0f / 536870912.0f, k21 = 1.0f / 2097152.0f, k22 = 4194304.0f;
     const float vx = (float)(int)(v.x >> 32) * k29, vy = (float)(int)(v.y >> 32) * k29;
     const long long wx = (v.x + 128) >> 8, wy = (v.y + 128) >> 8;  // 2^-53 pu
-    const float inv = __fdividef(1.0f, fmaf(vx, vx, vy * vy));
+    const float v2 = fmaf(vx, vx, vy * vy), inv = __fdividef(1.0f, v2);
     const float ix = fmaf(s_f.x, vx, s_f.y * vy) * inv, iy = fmaf(s_f.x, vy, -s_f.y * vx) * inv;
-    const bool ok = fabsf(ix) < 33554432.0f && fabsf(iy) < 33554432.0f;
+    const bool ok = fabsf(ix) < 33554432.0f && fabsf(iy) < 33554432.0f && v2 >= kLowV2;
     const int qx = __float2int_rn(ix), qy = __float2int_rn(iy);
     using u64 = unsigned long long;  // modulo 2^64
     auto mul = [](int q, long long w) { return (u64)(long long)q * (u64)w; };

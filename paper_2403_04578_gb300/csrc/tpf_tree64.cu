@@ -20,8 +20,8 @@
 // path sums and V integers of 2^-61 pu.  Integer sums are exact, so what an FP64 prefix sum loses at its
 // own magnitude is not lost; V is rounded to FP64 where it enters a product and where it is returned.
 // The block's largest step is taken in FP32 and repeated in FP64 when it lies within 1e-5 of tol.  A column
-// that leaves the range of the integers (a current beyond four times the largest load, a drop of half a pu
-// on one branch or of 1 pu in all, anything not finite) starts again in FP64 throughout.
+// that leaves the range of the integers (a voltage below half a pu, a current beyond four times the largest
+// load, a drop of half a pu on one branch or of 1 pu in all, anything not finite) starts again in FP64 throughout.
 //
 // One block owns one column for its whole solve, with the slot layout of the mixed kernel
 // (thread k owns depth-first positions k*bpt .. k*bpt + bpt - 1, position q at slot
@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
                         run = ladd(run, I);
                     } else {
                         const double2 I = demand64<kZip>(make_double2(from_fx(vi.x, -kFx), from_fx(vi.y, -kFx)), Ss[s], g, s);
-                        over |= order(I.x) >= cur_e || order(I.y) >= cur_e;
+                        over |= order(I.x) >= cur_e || order(I.y) >= cur_e || !(abs2_fx(vi) >= kLowV2);
                         run = ladd(run, make_longlong2(to_fx(I.x, -cur), to_fx(I.y, -cur)));
                     }
                 }
