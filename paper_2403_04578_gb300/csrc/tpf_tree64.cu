@@ -21,7 +21,8 @@
 // own magnitude is not lost; V is rounded to FP64 where it enters a product and where it is returned.
 // The block's largest step is taken in FP32 and repeated in FP64 when it lies within 1e-5 of tol.  A column
 // that leaves the range of the integers (a voltage below half a pu, a current beyond four times the largest
-// load, a drop of half a pu on one branch or of 1 pu in all, anything not finite) starts again in FP64 throughout.
+// load, a drop of half a pu on one branch or of 1 pu in all, anything not finite), or whose last place is too coarse
+// for the feeder's impedances (fixed_limits below), is solved in FP64 throughout.
 //
 // One block owns one column for its whole solve, with the slot layout of the mixed kernel
 // (thread k owns depth-first positions k*bpt .. k*bpt + bpt - 1, position q at slot
@@ -48,7 +49,8 @@ struct Tree64Args {
     float tol2_lo, tol2_hi;  // tol2 in units of 2^-122 less and plus 1e-5 of itself
     int fixed;       // sums in fixed point
     int log2n;       // n <= 2^log2n
-    int z_e;         // every component of z is below 2^z_e
+    int z_e;         // every component of z but the large ones is below 2^z_e
+    int cur_max;     // the coarsest last place of a column's currents (DeviceNet)
     longlong2 vs_fx; // slack voltage in 2^-61 pu
     double2 vs;      // slack voltage
     const int *col, *end, *par, *ecnt, *kidx;
@@ -224,14 +226,19 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
     const int cur_e = min(max((int)(smax >> 20) - 1022, -800), 1024) + 2, cur = cur_e + g.log2n - 62;
     // Branch terms z L: products in units of 2^(cur + z_e - 61) for a result in 2^-61 pu.
     const int zsh = min(-(cur + g.z_e), 126);
-    bool fixed = g.fixed && cur_e < 900 && zsh >= 1, over = false;
+    bool fixed = g.fixed && cur_e < 900 && zsh >= 1 && cur <= g.cur_max, over = false;
+    unsigned large = 0;  // the thread's positions with an impedance of 2^z_e and more
     if (fixed) {
 #pragma unroll
         for (int j = 0; j < kBPT; ++j) {
             over |= order(V[j].x) >= 1 || order(V[j].y) >= 1;
             set_v(j, make_longlong2(to_fx(V[j].x, kFx), to_fx(V[j].y, kFx)));
             const int s = j * th + tid;
-            const double2 zv = Zs[s];
+            double2 zv = Zs[s];
+            if (max(order(zv.x), order(zv.y)) >= g.z_e) {
+                large |= 1u << j;
+                zv = make_double2(0.0, 0.0);
+            }
             Zi[s] = make_longlong2(to_fx(zv.x, 61 - g.z_e), to_fx(zv.y, 61 - g.z_e));
             if (kInt) {
                 const int u = cur_e - 25;
@@ -282,6 +289,7 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
                     if (j) L = lsub(L, loc[j - 1]);
                     else if (q > 0) L = lsub(L, PXi[(kBPT - 1) * th + tid - 1]);
                     over |= !branch_fx(Zi[s], L, zsh, x);
+                    if (large & 1u << j) over |= (L.x | L.y) != 0;
                 }
                 loc[j] = x;
             }
@@ -582,6 +590,52 @@ int tree64_bpt(int n) {
     return 0;
 }
 
+// Which columns take the integers.  A column's currents are rounded to 2^cur, an error of 0.29 2^cur (root mean
+// square), and bus k's moves V_q by R_qk, the impedance that their paths share; impedances are rounded to
+// 2^(z_e - 61), which moves V_q by 0.29 2^(z_e - 61) times the current of each branch on its path, at most
+// 2^(cur + 62 - log2n) per bus below it.  Half a last place of V, 2^-54 pu, is allowed for both together, in root
+// mean square; the sums of squares grow along a path.  The feeders of inputs.py are 21 times below that (1,000
+// buses).  One load of thousands of times the others is not: such columns lost 3.3e-14 pu (1,000 pu beside 399
+// ordinary loads) to 3.0e-11 (1e6 pu).
+// Impedances above 2^8 times the median set neither z_e nor the limit, but a column with a current there goes to
+// FP64 (the kernel looks).  Most are open switches, without a current: a stub of 1e6 pu cost the others 7.4e-13 pu
+// when it set the place of all impedances, one of 1e12 pu 7.9e-7.
+void fixed_limits(const Network &net, int &z_e, int &cur_max) {
+    const int n = net.n_pq;
+    std::vector<int> e(n);
+    for (int q = 0; q < n; ++q) frexp(std::max(std::fabs(net.dfs_z[2 * q]), std::fabs(net.dfs_z[2 * q + 1])), &e[q]);
+    std::vector<int> by_size = e;
+    std::nth_element(by_size.begin(), by_size.begin() + n / 2, by_size.end());
+    const int cut = by_size[n / 2] + 8;
+    z_e = -2000;
+    for (int v : e)
+        if (v <= cut) z_e = std::max(z_e, v);
+    int log2n = 0;
+    while ((1 << log2n) < n) ++log2n;
+    struct At {
+        int end;              // of the subtree's positions
+        double re, im, sum;  // path impedance; both sums of squares over 0.29^2 4^cur
+    };
+    std::vector<At> path;  // the ancestors of position q
+    double worst = 0.0;
+    for (int q = 0; q < n; ++q) {
+        while (!path.empty() && path.back().end <= q) path.pop_back();
+        const At up = path.empty() ? At{n, 0.0, 0.0, 0.0} : path.back();
+        At a = up;
+        a.end = net.dfs_end[q];
+        if (e[q] <= cut) {
+            const double size = a.end - q, zq = std::ldexp(size, z_e + 1 - log2n);
+            a.re += net.dfs_z[2 * q];
+            a.im += net.dfs_z[2 * q + 1];
+            a.sum += size * ((a.re * a.re + a.im * a.im) - (up.re * up.re + up.im * up.im)) + zq * zq;
+        }
+        worst = std::max(worst, a.sum);
+        path.push_back(a);
+    }
+    const double c = std::log2(std::ldexp(1.0, -54) / (0.29 * std::sqrt(worst)));
+    cur_max = c >= 900.0 ? 900 : (c >= -900.0 ? (int)std::floor(c) : -10000);
+}
+
 tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t *iters, double *mismatch,
                         const tpf_opts &o, cudaStream_t st) {
     const DeviceNet &d = h->dev;
@@ -605,13 +659,8 @@ tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_
     g.tol2_hi = (float)(ldexp(g.tol2, 2 * kFx) * (1.0 + 1e-5));
     g.fixed = fabs(g.vs.x) < 2.0 && fabs(g.vs.y) < 2.0 && o.tol < 1.0;
     while ((1 << g.log2n) < d.n) ++g.log2n;
-    {
-        double zm = 0.0;
-        for (double c : h->net.dfs_z) zm = std::max(zm, std::fabs(c));
-        frexp(zm, &g.z_e);
-        if (!(zm < 1e30)) g.fixed = 0;
-        g.z_e = std::max(g.z_e, -60);
-    }
+    g.z_e = d.t64_z_e;
+    g.cur_max = d.t64_cur_max;
     if (g.fixed) g.vs_fx = make_longlong2(llrint(ldexp(g.vs.x, kFx)), llrint(ldexp(g.vs.y, kFx)));
     g.col = d.t_col;
     g.end = d.t_end;
