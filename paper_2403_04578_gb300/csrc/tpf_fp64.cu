@@ -78,7 +78,7 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
             std::vector<int> col64(ns64, -1), end64(ns64, 0), par64(ns64, -1), ecnt(ns64, 0), kidx(ns64, -1);
             d.t64_threads = th64;
             d.t64_bpt = bpt64;
-            if (ph == 1) fixed_limits(net, d.t64_z_e, d.t64_cur_max);
+            if (ph == 1) fixed_limits(net, d.t64_z_e, d.t64_cur_max, d.t64_cur_min);
             int n_ends = 0;  // entries of the ends lists laid out so far, in position order
             std::vector<float4> z(ns, make_float4(0.f, 0.f, 0.f, 0.f));
             std::vector<double2> z64(ph == 1 ? ns64 : 0, make_double2(0.0, 0.0)), y64 = z64;

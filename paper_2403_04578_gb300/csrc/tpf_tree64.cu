@@ -50,7 +50,8 @@ struct Tree64Args {
     int fixed;       // sums in fixed point
     int log2n;       // n <= 2^log2n
     int z_e;         // every component of z but the large ones is below 2^z_e
-    int cur_max;     // the coarsest last place of a column's currents (DeviceNet)
+    int cur_max;     // the coarsest last place of a column's currents, and the finest with which the
+    int cur_min;     // mismatch's branch currents still fit (DeviceNet)
     longlong2 vs_fx; // slack voltage in 2^-61 pu
     double2 vs;      // slack voltage
     const int *col, *end, *par, *ecnt, *kidx;
@@ -156,6 +157,9 @@ __device__ __forceinline__ int next_slot64(int s, int th) {
     return s < (kBPT - 1) * th ? s + th : s - (kBPT - 1) * th + 1;
 }
 
+// Beside the slot of a subtree's last position (below 4,096): the position's impedance is 2^z_e and more.
+constexpr int kLarge = 1 << 14;
+
 // Currents in integers up to 2,048 buses (8 B more of shared memory a slot than 4,096 buses leave).
 template <int kBPT>
 constexpr bool kIntCurrents = kBPT < 8;
@@ -227,7 +231,6 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
     // Branch terms z L: products in units of 2^(cur + z_e - 61) for a result in 2^-61 pu.
     const int zsh = min(-(cur + g.z_e), 126);
     bool fixed = g.fixed && cur_e < 900 && zsh >= 1 && cur <= g.cur_max, over = false;
-    unsigned large = 0;  // the thread's positions with an impedance of 2^z_e and more
     if (fixed) {
 #pragma unroll
         for (int j = 0; j < kBPT; ++j) {
@@ -236,7 +239,7 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
             const int s = j * th + tid;
             double2 zv = Zs[s];
             if (max(order(zv.x), order(zv.y)) >= g.z_e) {
-                large |= 1u << j;
+                s_rng[s] |= kLarge;
                 zv = make_double2(0.0, 0.0);
             }
             Zi[s] = make_longlong2(to_fx(zv.x, 61 - g.z_e), to_fx(zv.y, 61 - g.z_e));
@@ -284,12 +287,12 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
                 const int q = base + j, s = j * th + tid;
                 longlong2 x = make_longlong2(0, 0);
                 if (q < n) {
-                    const int ls = s_rng[s];
+                    const int rl = s_rng[s], ls = rl & (kLarge - 1);
                     longlong2 L = ls == s ? loc[j] : PXi[ls];
                     if (j) L = lsub(L, loc[j - 1]);
                     else if (q > 0) L = lsub(L, PXi[(kBPT - 1) * th + tid - 1]);
                     over |= !branch_fx(Zi[s], L, zsh, x);
-                    if (large & 1u << j) over |= (L.x | L.y) != 0;
+                    if (rl & kLarge) over |= (L.x | L.y) != 0;
                 }
                 loc[j] = x;
             }
@@ -342,6 +345,7 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
                     V[j] = q < n && g.given ? Vc[g.col[s]] : make_double2(1.0, 0.0);
                     if (kInt) Ss[s] = q < n ? S[g.col[s]] : make_double2(0.0, 0.0);
                     Zs[s] = q < n ? g.z[s] : make_double2(0.0, 0.0);
+                    s_rng[s] &= kLarge - 1;
                 }
                 continue;
             }
@@ -444,14 +448,30 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
     // the returned V (ZIP: |V_i| |(Y v)_i + i_d,i|).  On the tree (Y v)_q = -J_q + sum over the
     // children k of J_k with the branch currents J_k = y_k (V_parent(k) - V_k), y_k = 1 / z_k.
     // In fixed point the branch currents and their sums are integers of 2^cur like the load currents, and
-    // the largest mismatch is compared as a square.
+    // the largest mismatch is compared as a square.  The last place of the returned V times a very large y can be
+    // beyond those integers (cur_min): then FP64.
     double worst = 0.0;
     if (fixed) {
 #pragma unroll
         for (int j = 0; j < kBPT; ++j) {
-            const int q = base + j, s = j * th + tid;
             const longlong2 v = get_v(j);
             V[j] = make_double2(from_fx(v.x, -kFx), from_fx(v.y, -kFx));
+        }
+    }
+    if (fixed && g.mismatch_out && cur < g.cur_min) {
+        fixed = false;
+#pragma unroll 1
+        for (int j = 0; j < kBPT; ++j) {
+            const int q = base + j, s = j * th + tid;
+            if (kInt) Ss[s] = q < n ? S[g.col[s]] : make_double2(0.0, 0.0);
+            Zs[s] = q < n ? g.z[s] : make_double2(0.0, 0.0);
+            s_rng[s] &= kLarge - 1;
+        }
+    }
+    if (fixed) {
+#pragma unroll
+        for (int j = 0; j < kBPT; ++j) {
+            const int q = base + j, s = j * th + tid;
             if (q < n) Vc[g.col[s]] = V[j];
             PXi[s] = make_longlong2(to_fx(V[j].x, kFx), to_fx(V[j].y, kFx));  // the returned V, rounded to FP64
         }
@@ -479,10 +499,10 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
                 const int q = base + j, s = j * th + tid;
                 if (q >= n) continue;
                 longlong2 acc = make_longlong2(-J[j].x, -J[j].y);
-                const int lq = s_rng[s];
+                const int lq = s_rng[s] & (kLarge - 1);
                 for (int ks = lq == s ? -1 : next_slot64<kBPT>(s, th); ks >= 0;) {
                     acc = ladd(acc, PXi[ks]);
-                    const int lc = s_rng[ks];
+                    const int lc = s_rng[ks] & (kLarge - 1);
                     ks = lc == lq ? -1 : next_slot64<kBPT>(lc, th);
                 }
                 const double2 a = make_double2(from_fx(acc.x, cur), from_fx(acc.y, cur)), v = V[j];
@@ -600,7 +620,10 @@ int tree64_bpt(int n) {
 // Impedances above 2^8 times the median set neither z_e nor the limit, but a column with a current there goes to
 // FP64 (the kernel looks).  Most are open switches, without a current: a stub of 1e6 pu cost the others 7.4e-13 pu
 // when it set the place of all impedances, one of 1e12 pu 7.9e-7.
-void fixed_limits(const Network &net, int &z_e, int &cur_max) {
+// cur_min is for the mismatch alone: a bus's branch currents are off by up to 2^-50 sum |y| (V is returned to 2^-52
+// pu), and 2^61 integers hold that beside the currents.  Only branches of 1e-14 pu and less, or loads as small,
+// come near (the sums wrapped there, and the mismatch was reported as 16 instead of 29).
+void fixed_limits(const Network &net, int &z_e, int &cur_max, int &cur_min) {
     const int n = net.n_pq;
     std::vector<int> e(n);
     for (int q = 0; q < n; ++q) frexp(std::max(std::fabs(net.dfs_z[2 * q]), std::fabs(net.dfs_z[2 * q + 1])), &e[q]);
@@ -615,14 +638,20 @@ void fixed_limits(const Network &net, int &z_e, int &cur_max) {
     struct At {
         int end;              // of the subtree's positions
         double re, im, sum;  // path impedance; both sums of squares over 0.29^2 4^cur
+        int q;
     };
+    std::vector<double> y(n, 0.0);  // sum of |y| over the branches at a position
     std::vector<At> path;  // the ancestors of position q
     double worst = 0.0;
     for (int q = 0; q < n; ++q) {
         while (!path.empty() && path.back().end <= q) path.pop_back();
-        const At up = path.empty() ? At{n, 0.0, 0.0, 0.0} : path.back();
+        const At up = path.empty() ? At{n, 0.0, 0.0, 0.0, -1} : path.back();
         At a = up;
         a.end = net.dfs_end[q];
+        a.q = q;
+        const double yq = 1.0 / std::hypot(net.dfs_z[2 * q], net.dfs_z[2 * q + 1]);
+        y[q] += yq;
+        if (up.q >= 0) y[up.q] += yq;
         if (e[q] <= cut) {
             const double size = a.end - q, zq = std::ldexp(size, z_e + 1 - log2n);
             a.re += net.dfs_z[2 * q];
@@ -634,6 +663,8 @@ void fixed_limits(const Network &net, int &z_e, int &cur_max) {
     }
     const double c = std::log2(std::ldexp(1.0, -54) / (0.29 * std::sqrt(worst)));
     cur_max = c >= 900.0 ? 900 : (c >= -900.0 ? (int)std::floor(c) : -10000);
+    const double m = std::log2(*std::max_element(y.begin(), y.end())) - 111.0;
+    cur_min = m <= 900.0 ? (int)std::ceil(std::max(m, -10000.0)) : 10000;
 }
 
 tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t *iters, double *mismatch,
@@ -661,6 +692,7 @@ tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_
     while ((1 << g.log2n) < d.n) ++g.log2n;
     g.z_e = d.t64_z_e;
     g.cur_max = d.t64_cur_max;
+    g.cur_min = d.t64_cur_min;
     if (g.fixed) g.vs_fx = make_longlong2(llrint(ldexp(g.vs.x, kFx)), llrint(ldexp(g.vs.y, kFx)));
     g.col = d.t_col;
     g.end = d.t_end;
