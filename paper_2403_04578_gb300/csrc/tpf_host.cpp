@@ -412,6 +412,17 @@ void compute_dense(Network &net) {
 
 namespace {
 
+// Copies of page-locked (or managed, or device) memory run beside the host thread, those of other memory do not.
+bool overlaps(const void *p) {
+    if (!p) return true;
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type != cudaMemoryTypeUnregistered;
+}
+
 // The host-buffer solve: columns are independent, so it runs chunk by chunk on the device
 // workspace (see the comment inside); solve(cols, S_dev, V_dev, iters_dev, mismatch_dev) solves one
 // chunk on `stream` and leaves its statistics in h->stats.  v_in: V_host holds a start to copy in.
@@ -441,13 +452,18 @@ tpf_status host_chunks(tpf_handle *h, int64_t T, const void *S_host, void *V_hos
     // fill, drain and host round trip (100 us) not to count: sqrt(3 MB times all bytes), 16 MB at least and 32
     // chunks at most.  Pinned, 20,160 columns of 999 buses (322 MB each way) take 4.86 ms in one chunk, 2.66 in
     // chunks of 32 MB, 2.90 of 16 and 3.75 of 8; 5,000 columns 1.29 ms, 0.88 of 24, 0.90 of 16; 86,400 of 99
-    // buses 2.23, 1.39 of 32, 1.34 of 24, 1.68 of 8; 15 MB and less are one chunk (no difference).  The
-    // learned start predicts 128 columns per SM at a time and takes 16,384 columns at least; the dense
+    // buses 2.23, 1.39 of 32, 1.34 of 24, 1.68 of 8; 15 MB and less are one chunk (no difference).
+    // That needs results in page-locked memory, and loads too or else the counts and mismatches.  The driver copies
+    // other memory with the host thread, and into memory that has never been written (numpy.empty) very slowly
+    // beside a running solve: 20,160 columns of 999 buses, pageable, 6.0 ms by bytes and 5.1 in one chunk, into
+    // new memory 100 ms and 17.  Such buffers are cut from 65,536 columns on.
+    // The learned start predicts 128 columns per SM at a time and takes 16,384 columns at least; the dense
     // solve's per-sweep host loop prefers few chunks.
     const bool sparse = o.method == TPF_METHOD_SPARSE;
+    const bool async = overlaps(V_host) && (overlaps(S_host) || (overlaps(iters_host) && overlaps(mismatch_host)));
     const double bytes = (double)T * (double)col_bytes, least = 16e6;
     int64_t n_chunks = 1;
-    if (sparse && !wide)
+    if (sparse && !wide && async)
         n_chunks = std::max<int64_t>(1, std::min<int64_t>(32, (int64_t)(bytes / std::max(least, std::sqrt(3e6 * bytes)))));
     else if (T >= 65536)
         n_chunks = std::min<int64_t>(sparse ? 32 : 8, T / 16384);
