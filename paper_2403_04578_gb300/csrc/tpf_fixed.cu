@@ -661,15 +661,20 @@ tpf_status solve_fixed(tpf_handle *h, int64_t T, const void *S, void *V, const t
     const int k_order = d.k_order;  // every component of K / c is below 2^k_order
     int64_t launches = 0, gemms = 0, gemm_cols = 0;
     if (!d.Kd16) {
-        if (cudaMalloc(&d.Kd16, sizeof(__half) * 2 * kDig * plane_k) != cudaSuccess) {
+        __half *planes = nullptr;
+        if (cudaMalloc(&planes, sizeof(__half) * 2 * kDig * plane_k) != cudaSuccess) {
             cudaGetLastError();
-            d.Kd16 = nullptr;
             return TPF_ENOMEM;
         }
         fx_k_digits<<<(unsigned)((plane_k + 255) / 256), 256, 0, st>>>((const double2 *)d.K64, d.k_col_order, n, n_pad,
-                                                                       kBits - k_order, (__half *)d.Kd16,
-                                                                       (__half *)d.Kd16 + kDig * plane_k);
-        TPF_CK(cudaGetLastError());
+                                                                       kBits - k_order, planes, planes + kDig * plane_k);
+        // The handle has them once they are written: its next solve may be on another stream.
+        if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(planes);
+            return TPF_ECUDA;
+        }
+        d.Kd16 = planes;
         ++launches;
     }
     int sms = 0;

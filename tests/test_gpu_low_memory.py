@@ -1,0 +1,68 @@
+"""Solves that meet a full device: TPF_ENOMEM or another way to the same result, and a handle that works afterwards.
+
+The rest of the device's memory is held in one allocation while a call runs.  Kernels that the call may take have
+run before, so that nothing but the library's buffers is allocated in between.
+"""
+import contextlib
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2403_04578_gb300 import inputs as G  # noqa: E402
+from paper_2403_04578_gb300 import tpf  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+MB = 1 << 20
+# Bounds the difference of two kernels' results: n 2^-53 times a drop of 0.05 pu, n = 999, and the map contracts.
+BOUND = 2e-14
+
+
+@contextlib.contextmanager
+def _leave(bytes_):
+    """At most about `bytes_` of device memory left inside."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    held = []
+    for step in (1 << 30, 32 * MB, 2 * MB):
+        while torch.cuda.mem_get_info()[0] >= bytes_ + step:
+            n = (torch.cuda.mem_get_info()[0] - bytes_) // step * step
+            held.append(torch.empty(n, dtype=torch.uint8, device="cuda"))
+    try:
+        yield
+    finally:
+        torch.cuda.synchronize()
+        held.clear()
+        torch.cuda.empty_cache()
+
+
+def _warm(T):
+    """Every FP64 dense kernel has run; the loads and outputs of a 999-bus solve, and its handle with K in place."""
+    for n in (10, 40):
+        f = G.make_feeder(n, 1)
+        with tpf.Feeder.from_inputs(f) as fd:
+            fd.solve(torch.from_numpy(G.load_tensor(f, 8, 1)).cuda(), precision="fp64", method="dense")
+    f = G.make_feeder(1000, 1)
+    S = torch.from_numpy(np.ascontiguousarray(G.load_tensor(f, T, 3))).cuda()
+    fd = tpf.Feeder.from_inputs(f)
+    fd.solve(S, precision="mixed", method="dense", tol=1e-10)
+    return fd, S, (torch.empty_like(S), torch.empty(T, dtype=torch.int32, device="cuda"),
+                   torch.empty(T, dtype=torch.float64, device="cuda"))
+
+
+# K's digit planes take 29 MB; those of 2,000 columns' currents 88 MB.
+@pytest.mark.parametrize("T,left", [(64, 20 * MB), (2000, 72 * MB)])
+def test_solve_after_a_full_device(T, left):
+    fd, S, (V, it, mm) = _warm(T)
+    with fd:
+        with _leave(left):
+            try:
+                fd.solve(S, V=V, iters=it, mismatch=mm, precision="fp64", method="dense", tol=1e-10)
+            except tpf.TpfError as e:
+                assert e.status == tpf.ENOMEM
+        other = torch.cuda.Stream()
+        V2, it2, _, st = fd.solve(S, precision="fp64", method="dense", tol=1e-10, stream=other)
+        Vs, its, _, _ = fd.solve(S, precision="fp64", method="sparse", tol=1e-10)
+    assert st == tpf.OK and bool((it2 == its).all())
+    assert float((V2 - Vs).abs().max()) <= BOUND
