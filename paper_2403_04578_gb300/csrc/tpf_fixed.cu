@@ -648,7 +648,8 @@ struct FxEvents {
 // From 17 demand buses on: up to 16 the FP64 kernel takes a single chunk of K per tile and both sides wait
 // for launches (3 to 10 buses: 260 to 390 us with FP64 FMAs, 276 to 410 here; 19 buses x 96 columns 573
 // against 394, 33 x 1,440 905 against 514, 199 x 288 4,516 against 939, 199 x 8,760 26,540 against 1,950,
-// 999 x 2,000 109.5 ms against 3.9).  Past 8,192 a column's currents no longer fit fx_slice's shared memory.
+// 999 x 2,000 109.5 ms against 3.9).  Without room for the digit planes (28 n_pad^2 bytes of K, at most 104 MB of
+// currents) solve_fixed returns TPF_ENOMEM before it touches V, and the FP64 kernel serves the call.  Past 8,192 a column's currents no longer fit fx_slice's shared memory.
 bool use_fixed(int n, int64_t T) { return n > 16 && n <= kFxMaxN && T < ((int64_t)1 << 31) - kFxN; }
 
 tpf_status solve_fixed(tpf_handle *h, int64_t T, const void *S, void *V, const tpf_opts &o, cudaStream_t st,
@@ -693,6 +694,8 @@ tpf_status solve_fixed(tpf_handle *h, int64_t T, const void *S, void *V, const t
         w.fx_bytes = 0;
         if (cudaMalloc(&w.fx_buf, need) != cudaSuccess) {
             cudaGetLastError();
+            cudaFree(d.Kd16);  // leaves the room to the FP64 sweeps
+            w.fx_buf = d.Kd16 = nullptr;
             return TPF_ENOMEM;
         }
         w.fx_bytes = need;

@@ -6,7 +6,7 @@
 // rule).  Here each sweep is one kernel over (64-bus x 32-column) output tiles: the tile's injections
 // conj(S ./ V) are formed from V_k in shared memory chunk by chunk (the Hadamard step of Algorithm 1),
 // multiplied by the matching K tile with FP64 FMAs, W is added and the per-column max |V_{k+1} - V_k| is
-// folded in with an atomic max.  It also serves the allocation-free solve, which has no room for digit
+// folded in with an atomic max.  It also serves the allocation-free solve, and solves without room for digit
 // planes.
 #include <algorithm>
 #include <cstdio>
@@ -697,7 +697,7 @@ tpf_status solve_fp64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t 
                       const tpf_opts &o, cudaStream_t st) {
     tpf_status rs = ensure_dense(h);
     if (rs != TPF_OK) return rs;
-    const bool fixed = use_fixed(h->dev.n, T);
+    bool fixed = use_fixed(h->dev.n, T);
     rs = ensure_workspace(h, T, fixed ? kWsState : kWsFp64);
     if (rs != TPF_OK) return rs;
     Workspace &w = h->ws;
@@ -708,8 +708,13 @@ tpf_status solve_fp64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t 
     KernelTimer timer(o.profile != 0, st);
     if (fixed) {
         rs = solve_fixed(h, T, S, V, o, st, timer, &sweeps, &launches, &gemms, &gemm_cols);
+        if (rs == TPF_ENOMEM) {  // no room for its digit planes
+            fixed = false;
+            rs = ensure_workspace(h, T, kWsFp64);
+        }
         if (rs != TPF_OK) return rs;
-    } else {
+    }
+    if (!fixed) {
         TPF_CK(cudaMemsetAsync(w.counters, 0, sizeof(int) * 8, st));
         {
             int64_t work = cols > T * n ? cols : T * n;

@@ -58,7 +58,8 @@ def test_solve_after_a_full_device(T, left):
     with fd:
         with _leave(left):
             try:
-                fd.solve(S, V=V, iters=it, mismatch=mm, precision="fp64", method="dense", tol=1e-10)
+                fd.solve(S, V=V, iters=it, mismatch=mm, start="flat", precision="fp64",
+                         method="dense", tol=1e-10)
             except tpf.TpfError as e:
                 assert e.status == tpf.ENOMEM
         other = torch.cuda.Stream()
@@ -66,3 +67,18 @@ def test_solve_after_a_full_device(T, left):
         Vs, its, _, _ = fd.solve(S, precision="fp64", method="sparse", tol=1e-10)
     assert st == tpf.OK and bool((it2 == its).all())
     assert float((V2 - Vs).abs().max()) <= BOUND
+
+
+@pytest.mark.parametrize("T,left", [(64, 20 * MB), (2000, 72 * MB)])
+def test_fp64_dense_without_room_for_digit_planes(T, left):
+    fd, S, (V, it, mm) = _warm(T)
+    with fd:
+        with _leave(left):
+            _, _, _, st = fd.solve(S, V=V, iters=it, mismatch=mm, start="flat", precision="fp64",
+                                   method="dense", tol=1e-10)
+            plain = fd.stats()["kernel_launches"]
+        V2, it2, mm2, st2 = fd.solve(S, precision="fp64", method="dense", tol=1e-10)
+        assert fd.stats()["kernel_launches"] > plain  # four kernels a sweep instead of two
+    assert st == st2 == tpf.OK and bool((it == it2).all())
+    assert float((V - V2).abs().max()) <= BOUND
+    assert float(mm.max()) <= 1e-8 and float(mm2.max()) <= 1e-8
