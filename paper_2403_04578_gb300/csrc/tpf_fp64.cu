@@ -166,6 +166,7 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
                        !up(&d.t_zf, zf) ||
                        (ph == 1 && (!up(&d.t_z64, z64) || !up(&d.t_y64, y64))) || (ph > 1 && (!up(&d.t_zrow, zrow) || !up(&d.t_yrow, yrow) || !up(&d.t_zrow_f, zrow_f)))) {
                 cudaGetLastError();
+                d.t_threads = 0;  // no layout
                 return TPF_ECUDA;
             }
         }
@@ -303,9 +304,8 @@ static tpf_status upload_column_orders(tpf_handle *h) {
     return TPF_OK;
 }
 
-tpf_status ensure_dense(tpf_handle *h) {
+static tpf_status build_dense(tpf_handle *h) {
     DeviceNet &d = h->dev;
-    if (d.K64) return TPF_OK;
     Network &net = h->net;
     try {
         compute_dense(net);
@@ -336,7 +336,49 @@ tpf_status ensure_dense(tpf_handle *h) {
                                                           (__half *)d.Kr16, (__half *)d.Ki16);
     TPF_CK(cudaGetLastError());
     TPF_CK(cudaDeviceSynchronize());
-    std::vector<double>().swap(net.K);  // the device copies serve from here on
+    return TPF_OK;
+}
+
+tpf_status ensure_dense(tpf_handle *h) {
+    DeviceNet &d = h->dev;
+    if (d.K64) return TPF_OK;
+    const tpf_status rs = build_dense(h);
+    if (rs != TPF_OK) {  // all or nothing: K64 says that everything is there
+        cudaFree(d.K64); cudaFree(d.W64); cudaFree(d.Kr16); cudaFree(d.Ki16);
+        d.K64 = d.W64 = nullptr;
+        d.Kr16 = d.Ki16 = nullptr;
+        cudaGetLastError();
+        return rs;
+    }
+    std::vector<double>().swap(h->net.K);  // the device copies serve from here on
+    return TPF_OK;
+}
+
+static tpf_status upload_zip(tpf_handle *h, const double *alpha) {
+    DeviceNet &d = h->dev;
+    const int n = d.n;
+    TPF_CK(cudaMalloc(&d.zip64, sizeof(double) * 3 * (size_t)n));
+    TPF_CK(cudaMemcpy(d.zip64, alpha, sizeof(double) * 3 * (size_t)n, cudaMemcpyHostToDevice));
+    if (d.t_threads > 0) {
+        const int th = d.t_threads, bpt = d.t_bpt, ns = th * bpt;
+        std::vector<float4> hi(ns, make_float4(0.f, 0.f, 0.f, 0.f)), lo = hi;
+        const Network &net = h->net;
+        for (int q = 0; q < n; ++q) {
+            const int s = (q % bpt) * th + q / bpt, i = net.dfs_col[q];
+            float hv[3], lv[3];
+            for (int k = 0; k < 3; ++k) {
+                const double a = alpha[(size_t)k * n + i];
+                hv[k] = (float)a;
+                lv[k] = (float)(a - (double)hv[k]);
+            }
+            hi[s] = make_float4(hv[0], hv[1], hv[2], 0.f);
+            lo[s] = make_float4(lv[0], lv[1], lv[2], 0.f);
+        }
+        TPF_CK(cudaMalloc(&d.t_zip_hi, sizeof(float4) * ns));
+        TPF_CK(cudaMalloc(&d.t_zip_lo, sizeof(float4) * ns));
+        TPF_CK(cudaMemcpy(d.t_zip_hi, hi.data(), sizeof(float4) * ns, cudaMemcpyHostToDevice));
+        TPF_CK(cudaMemcpy(d.t_zip_lo, lo.data(), sizeof(float4) * ns, cudaMemcpyHostToDevice));
+    }
     return TPF_OK;
 }
 
@@ -364,30 +406,14 @@ tpf_status set_zip(tpf_handle *h, const double *alpha) {
     d.zip64 = nullptr;
     d.t_zip_hi = d.t_zip_lo = nullptr;
     if (!alpha) return TPF_OK;
-    const int n = d.n;
-    TPF_CK(cudaMalloc(&d.zip64, sizeof(double) * 3 * (size_t)n));
-    TPF_CK(cudaMemcpy(d.zip64, alpha, sizeof(double) * 3 * (size_t)n, cudaMemcpyHostToDevice));
-    if (d.t_threads > 0) {
-        const int th = d.t_threads, bpt = d.t_bpt, ns = th * bpt;
-        std::vector<float4> hi(ns, make_float4(0.f, 0.f, 0.f, 0.f)), lo = hi;
-        const Network &net = h->net;
-        for (int q = 0; q < n; ++q) {
-            const int s = (q % bpt) * th + q / bpt, i = net.dfs_col[q];
-            float hv[3], lv[3];
-            for (int k = 0; k < 3; ++k) {
-                const double a = alpha[(size_t)k * n + i];
-                hv[k] = (float)a;
-                lv[k] = (float)(a - (double)hv[k]);
-            }
-            hi[s] = make_float4(hv[0], hv[1], hv[2], 0.f);
-            lo[s] = make_float4(lv[0], lv[1], lv[2], 0.f);
-        }
-        TPF_CK(cudaMalloc(&d.t_zip_hi, sizeof(float4) * ns));
-        TPF_CK(cudaMalloc(&d.t_zip_lo, sizeof(float4) * ns));
-        TPF_CK(cudaMemcpy(d.t_zip_hi, hi.data(), sizeof(float4) * ns, cudaMemcpyHostToDevice));
-        TPF_CK(cudaMemcpy(d.t_zip_lo, lo.data(), sizeof(float4) * ns, cudaMemcpyHostToDevice));
+    const tpf_status rs = upload_zip(h, alpha);
+    if (rs != TPF_OK) {  // constant power again
+        cudaFree(d.zip64); cudaFree(d.t_zip_hi); cudaFree(d.t_zip_lo);
+        d.zip64 = nullptr;
+        d.t_zip_hi = d.t_zip_lo = nullptr;
+        cudaGetLastError();
     }
-    return TPF_OK;
+    return rs;
 }
 
 void free_device(tpf_handle *h) {
@@ -423,9 +449,9 @@ tpf_status ensure_workspace(tpf_handle *h, int64_t cols, int kind) {
     cols = round_up(cols, kTileN);
     const bool have_mixed = w.Vhi != nullptr;
     const bool have_fp64 = w.Valt != nullptr;
+    if (w.counters_host == nullptr) TPF_CK(cudaMallocHost(&w.counters_host, sizeof(int) * 16));
     if (w.counters == nullptr) {
         TPF_CK(cudaMalloc(&w.counters, sizeof(int) * 8));
-        TPF_CK(cudaMallocHost(&w.counters_host, sizeof(int) * 16));
         TPF_CK(cudaMemset(w.counters, 0, sizeof(int) * 8));
     }
     if (cols <= w.cap_cols && (mixed ? have_mixed : (fp64 ? have_fp64 : true))) return TPF_OK;
@@ -433,6 +459,7 @@ tpf_status ensure_workspace(tpf_handle *h, int64_t cols, int kind) {
     bool want_mixed = mixed || (have_mixed && cap > w.cap_cols);
     bool want_fp64 = fp64 || (have_fp64 && cap > w.cap_cols);
     if (cap > w.cap_cols) {
+        w.cap_cols = 0;  // until all of them are there
         cudaFree(w.delta_bits); cudaFree(w.delta64); cudaFree(w.iters); cudaFree(w.flags); cudaFree(w.rexp);
         cudaFree(w.tile_active); cudaFree(w.dprev);
         w.delta_bits = nullptr; w.delta64 = nullptr; w.iters = nullptr; w.flags = nullptr; w.rexp = nullptr;
@@ -467,6 +494,9 @@ tpf_status ensure_workspace(tpf_handle *h, int64_t cols, int kind) {
             cudaMalloc(&w.RefHi, sizeof(float2) * el) != cudaSuccess || cudaMalloc(&w.RefLo, sizeof(float2) * el) != cudaSuccess ||
             cudaMalloc(&w.Rr16, sizeof(__half) * el) != cudaSuccess || cudaMalloc(&w.Ri16, sizeof(__half) * el) != cudaSuccess) {
             cudaGetLastError();
+            cudaFree(w.Vhi); cudaFree(w.Vlo); cudaFree(w.Shi); cudaFree(w.Rr16); cudaFree(w.Ri16);
+            cudaFree(w.RefHi); cudaFree(w.RefLo);
+            w.Vhi = w.Vlo = w.Shi = w.RefHi = w.RefLo = nullptr; w.Rr16 = w.Ri16 = nullptr;  // Vhi says that all are there
             return TPF_ENOMEM;
         }
     }

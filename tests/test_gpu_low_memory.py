@@ -82,3 +82,37 @@ def test_fp64_dense_without_room_for_digit_planes(T, left):
     assert st == st2 == tpf.OK and bool((it == it2).all())
     assert float((V - V2).abs().max()) <= BOUND
     assert float(mm.max()) <= 1e-8 and float(mm2.max()) <= 1e-8
+
+
+def _expect_error(call):
+    with pytest.raises(tpf.TpfError) as e:
+        call()
+    assert e.value.status in (tpf.ENOMEM, tpf.ECUDA)
+
+
+def test_dense_form_after_a_full_device():
+    # K (16 MB) is built by the first dense solve, which fails; the next one has to build all of it.
+    f = G.make_feeder(1000, 1)
+    S = torch.from_numpy(np.ascontiguousarray(G.load_tensor(f, 64, 3))).cuda()
+    _warm(64)[0].close()
+    with tpf.Feeder.from_inputs(f) as fd:
+        Vs, its, _, _ = fd.solve(S, precision="fp64", method="sparse", tol=1e-10)
+        for left in (8 * MB, 20 * MB):
+            with _leave(left):
+                _expect_error(lambda: fd.solve(S, precision="mixed", method="dense", tol=1e-10))
+        V, it, _, st = fd.solve(S, precision="mixed", method="dense", tol=1e-10)
+    assert st == tpf.OK and bool((it > 0).all())
+    assert float((V - Vs).abs().max()) <= 1e-8  # the mixed path's bound
+
+
+def test_workspace_after_a_full_device():
+    # 20,000 columns need seven planes of 82 to 164 MB; the second one finds no room.
+    fd, S, _ = _warm(128)
+    with fd:
+        V, it, _, _ = fd.solve(S, precision="mixed", method="dense", tol=1e-10)
+        big = S.repeat(157, 1)[:20_000].contiguous()
+        out = torch.empty_like(big)
+        with _leave(240 * MB):
+            _expect_error(lambda: fd.solve(big, V=out, start="flat", precision="mixed", method="dense", tol=1e-10))
+        V2, it2, _, st = fd.solve(S, precision="mixed", method="dense", tol=1e-10)
+    assert st == tpf.OK and torch.equal(V, V2) and torch.equal(it, it2)
