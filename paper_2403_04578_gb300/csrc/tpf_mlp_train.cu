@@ -126,8 +126,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_gemm(const __grid_constant__ 
         n0 = (tile / g.m_tiles[p]) * kN;
         c1 = g.chunks;
     } else {
-        m0 = (int)blockIdx.x * kTileM;
-        n0 = (int)blockIdx.y * kN;
+        m0 = (int)blockIdx.y * kTileM;
+        n0 = (int)blockIdx.x * kN;
         c1 = g.chunks;
     }
 
@@ -369,14 +369,14 @@ __global__ void __launch_bounds__(256)
     mlp_features(const double2 *__restrict__ S, int B, int n, int P, int bus_tiles, const float *__restrict__ mean,
                  const float *__restrict__ sd, bf16 *X, bf16 *XT, int *err, double *loss) {
     __shared__ unsigned short s[2][32][34];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b0 = (int)blockIdx.y * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b0 = (int)blockIdx.x * 32, part = (int)blockIdx.y;
     after_predecessor();
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
         *err = 0;
         *loss = 0.0;
     }
-    if ((int)blockIdx.x >= bus_tiles) {  // padding features 2n .. P - 1
-        const int j0 = ((int)blockIdx.x - bus_tiles) * 32;
+    if (part >= bus_tiles) {  // padding features 2n .. P - 1
+        const int j0 = (part - bus_tiles) * 32;
         for (int r = ty; r < 32; r += 8) {
             const bf16 z = __float2bfloat16_rn(0.0f);
             if (2 * n + j0 + tx < P) X[(int64_t)(b0 + r) * P + 2 * n + j0 + tx] = z;
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(256)
         }
         return;
     }
-    const int j0 = (int)blockIdx.x * 32, j = j0 + tx;
+    const int j0 = part * 32, j = j0 + tx;
     if (j < n) {
         const float mr = mean[j], dr = sd[j], mi = mean[n + j], di = sd[n + j];
         double2 in[4];
@@ -450,7 +450,7 @@ tpf_status launch_layer(int kind, const LayerArgs &g, cudaStream_t st) {
                    big_smem(mlp_gemm<kTrainN, kBackward, LayerArgs>, R::kSmem);
         }))
         return TPF_ECUDA;
-    const dim3 grid((unsigned)(g.M / kTileM), (unsigned)(g.B / kTrainN));
+    const dim3 grid((unsigned)(g.B / kTrainN), (unsigned)(g.M / kTileM));  // y is limited to 65,535
     if (kind == kHidden) return launch_pdl(mlp_gemm<kTrainN, kHidden, LayerArgs>, grid, kThreads, R::kSmem, st, g);
     if (kind == kOutput) return launch_pdl(mlp_gemm<kTrainN, kOutput, LayerArgs>, grid, kThreads, R::kSmem, st, g);
     return launch_pdl(mlp_gemm<kTrainN, kBackward, LayerArgs>, grid, kThreads, R::kSmem, st, g);
@@ -476,7 +476,7 @@ tpf_status launch_adam(AdamArgs &g, cudaStream_t st) {
 tpf_status launch_train_features(const double2 *S, int B, int n, int P, const float *mean, const float *sd, bf16 *X,
                                  bf16 *XT, int *err, double *loss, cudaStream_t st) {
     const int bus_tiles = (n + 31) / 32, pad_tiles = (P - 2 * n + 31) / 32;
-    return launch_pdl(mlp_features, dim3((unsigned)(bus_tiles + pad_tiles), (unsigned)(B / 32)), 256, 0, st, S, B, n, P,
+    return launch_pdl(mlp_features, dim3((unsigned)(B / 32), (unsigned)(bus_tiles + pad_tiles)), 256, 0, st, S, B, n, P,
                       bus_tiles, mean, sd, X, XT, err, loss);
 }
 
