@@ -72,13 +72,13 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
             const int ph = net.phases, nb = n / ph;
             std::vector<int> col(ns, -1), end(ns, 0), par(ns, -1);
             // The FP64 sparse kernel's own layout (its sums are exact, so its results do not depend on it).
-            const int bpt64 = bpt == kTreeBigBPT ? bpt : tree64_bpt(n), th64 = bpt64 == bpt ? th : tree_threads(n, bpt64);
+            d.t64_fixed = ph == 1 && fixed_limits(net, d.t64_z_e, d.t64_cur_max, d.t64_cur_min);
+            const int bpt64 = bpt == kTreeBigBPT ? bpt : tree64_bpt(n, d.t64_fixed), th64 = bpt64 == bpt ? th : tree_threads(n, bpt64);
             const int ns64 = th64 * bpt64;
             auto slot64 = [th64, bpt64](int q) { return (q % bpt64) * th64 + q / bpt64; };
             std::vector<int> col64(ns64, -1), end64(ns64, 0), par64(ns64, -1), ecnt(ns64, 0), kidx(ns64, -1);
             d.t64_threads = th64;
             d.t64_bpt = bpt64;
-            if (ph == 1) fixed_limits(net, d.t64_z_e, d.t64_cur_max, d.t64_cur_min);
             int n_ends = 0;  // entries of the ends lists laid out so far, in position order
             std::vector<float4> z(ns, make_float4(0.f, 0.f, 0.f, 0.f));
             std::vector<double2> z64(ph == 1 ? ns64 : 0, make_double2(0.0, 0.0)), y64 = z64;

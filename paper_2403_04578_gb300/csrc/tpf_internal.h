@@ -134,7 +134,8 @@ struct DeviceNet {
     int t_threads = 0, t_bpt = 0;
     // t_col to t_kidx, t_z64 and t_y64 are the FP64 sparse kernel's, laid out for its own block shape.
     int t64_threads = 0, t64_bpt = 0;
-    int t64_z_e = 0, t64_cur_max = 0, t64_cur_min = 0;  // its integers' limits (fixed_limits, tpf_tree64.cu)
+    bool t64_fixed = false;  // its integers can serve, and their limits (fixed_limits, tpf_tree64.cu)
+    int t64_z_e = 0, t64_cur_max = 0, t64_cur_min = 0;
     int *t_col = nullptr, *t_end = nullptr, *t_par = nullptr, *t_ecnt = nullptr;
     int *t_kidx = nullptr;  // per slot: the index in ends order at which its position appears, or -1
     float4 *t_z = nullptr;
@@ -331,8 +332,8 @@ tpf_status solve_sparse_ex(tpf_handle *h, int64_t T, const void *S, void *V, int
 tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t *iters,
                         double *mismatch, const tpf_opts &o, cudaStream_t st);
 size_t tree64_smem(int threads, int bpt);
-int tree64_bpt(int n);
-void fixed_limits(const Network &net, int &z_e, int &cur_max, int &cur_min);
+int tree64_bpt(int n, bool fixed);
+bool fixed_limits(const Network &net, int &z_e, int &cur_max, int &cur_min);
 tpf_status solve_batch_sparse(int F, tpf_handle *const *hs, const int64_t *T, const void *const *S,
                               void *const *V, int32_t *const *iters, double *const *mismatch,
                               const tpf_opts &o, int64_t *conv_out, tpf_stats *stats, cudaStream_t st);

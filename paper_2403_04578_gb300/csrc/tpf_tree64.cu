@@ -603,10 +603,11 @@ size_t tree64_smem(int threads, int bpt) {
 // Buses per thread: two up to 512 buses (256 threads), where a thread's chain of sums and products is what a
 // column waits for; four up to 2,048, eight beyond (32 B of prefix sums and loads a slot).  In us, two against
 // four: 33 buses x 16,384 columns 196 and 389, 64 buses 228 and 434, 129 x 8,000 333 and 497, 299 buses 572 and 699,
-// 512 buses 865 and 872, 699 buses 1,487 and 1,287.
-int tree64_bpt(int n) {
+// 512 buses 865 and 872, 699 buses 1,487 and 1,287.  In FP64 throughout a thread's scans cost more than the chain:
+// 199 buses x 4,096 columns behind a source of 12.66 (kV) take 1,615 us at two and 1,345 at four.
+int tree64_bpt(int n, bool fixed) {
     for (int b : {2, 4, 8})
-        if ((b > 2 || n <= 512) && tree_threads(n, b)) return b;
+        if ((b > 2 || (fixed && n <= 512)) && tree_threads(n, b)) return b;
     return 0;
 }
 
@@ -623,7 +624,8 @@ int tree64_bpt(int n) {
 // cur_min is for the mismatch alone: a bus's branch currents are off by up to 2^-50 sum |y| (V is returned to 2^-52
 // pu), and 2^61 integers hold that beside the currents.  Only branches of 1e-14 pu and less, or loads as small,
 // come near (the sums wrapped there, and the mismatch was reported as 16 instead of 29).
-void fixed_limits(const Network &net, int &z_e, int &cur_max, int &cur_min) {
+// Returns false where no column of the feeder can take them: V is 61 bits below 2 pu, and none of it below 0.5.
+bool fixed_limits(const Network &net, int &z_e, int &cur_max, int &cur_min) {
     const int n = net.n_pq;
     std::vector<int> e(n);
     for (int q = 0; q < n; ++q) frexp(std::max(std::fabs(net.dfs_z[2 * q]), std::fabs(net.dfs_z[2 * q + 1])), &e[q]);
@@ -665,6 +667,8 @@ void fixed_limits(const Network &net, int &z_e, int &cur_max, int &cur_min) {
     cur_max = c >= 900.0 ? 900 : (c >= -900.0 ? (int)std::floor(c) : -10000);
     const double m = std::log2(*std::max_element(y.begin(), y.end())) - 111.0;
     cur_min = m <= 900.0 ? (int)std::ceil(std::max(m, -10000.0)) : 10000;
+    return std::fabs(net.vs_re) < 2.0 && std::fabs(net.vs_im) < 2.0 && std::hypot(net.vs_re, net.vs_im) >= 0.5 &&
+           cur_max > -10000;
 }
 
 tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t *iters, double *mismatch,
@@ -688,7 +692,7 @@ tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_
     g.vs = make_double2(h->net.vs_re, h->net.vs_im);
     g.tol2_lo = (float)(ldexp(g.tol2, 2 * kFx) * (1.0 - 1e-5));
     g.tol2_hi = (float)(ldexp(g.tol2, 2 * kFx) * (1.0 + 1e-5));
-    g.fixed = fabs(g.vs.x) < 2.0 && fabs(g.vs.y) < 2.0 && o.tol < 1.0;
+    g.fixed = d.t64_fixed && o.tol < 1.0;
     while ((1 << g.log2n) < d.n) ++g.log2n;
     g.z_e = d.t64_z_e;
     g.cur_max = d.t64_cur_max;
