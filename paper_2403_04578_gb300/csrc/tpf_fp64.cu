@@ -45,22 +45,75 @@ __global__ void k_to_fp16(const double *__restrict__ K, int n, int n_pad, float 
 
 // Slot-ordered depth-first arrays of the sparse formulation for blocks of tree_threads(n, bpt)
 // threads with bpt positions each (replacing any earlier layout; bpt 0 disables the sparse path).
+namespace {
+
+template <class P, class V>
+bool up(P **dst, const V &v) {
+    if (cudaMalloc((void **)dst, sizeof(P) * v.size()) != cudaSuccess) return false;
+    return cudaMemcpy(*dst, v.data(), sizeof(P) * v.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+}
+
+// Parent position of each depth-first position, -1 = the slack.
+std::vector<int> parent_positions(const Network &net) {
+    std::vector<int> par(net.n_pq, -1);
+    for (int q = 0; q < net.n_pq; ++q)
+        for (int c = q + 1; c < net.dfs_end[q]; c = net.dfs_end[c]) par[c] = q;
+    return par;
+}
+
+}  // namespace
+
+void free_tree64(Tree64 &t) {
+    cudaFree(t.col); cudaFree(t.end); cudaFree(t.par); cudaFree(t.ecnt); cudaFree(t.kidx); cudaFree(t.z); cudaFree(t.y);
+    t = Tree64();
+}
+
+tpf_status layout_tree64(const Network &net, int bpt, Tree64 &out) {
+    const int n = net.n_pq, th = tree_threads(n, bpt), ns = th * bpt;
+    auto slot = [th, bpt](int q) { return (q % bpt) * th + q / bpt; };
+    std::vector<int> col(ns, -1), end(ns, 0), par(ns, -1), ecnt(ns, 0), kidx(ns, -1);
+    std::vector<double2> z(ns, make_double2(0.0, 0.0)), y = z;
+    const std::vector<int> pos_par = parent_positions(net);
+    int n_ends = 0;  // entries of the ends lists laid out so far, in position order
+    for (int q = 0; q < n; ++q) {
+        const int s = slot(q);
+        col[s] = net.dfs_col[q];
+        end[s] = net.dfs_end[q];
+        par[s] = pos_par[q] < 0 ? -1 : slot(pos_par[q]);
+        ecnt[s] = n_ends | (net.dfs_eptr[q + 1] - net.dfs_eptr[q]) << 16;  // start | count << 16
+        for (int k = net.dfs_eptr[q]; k < net.dfs_eptr[q + 1]; ++k)
+            kidx[slot(net.dfs_ends[k])] = n_ends++;  // where its branch term is scattered
+        const double2 zq = make_double2(net.dfs_z[2 * q], net.dfs_z[2 * q + 1]);
+        const double z2 = zq.x * zq.x + zq.y * zq.y;
+        z[s] = zq;
+        y[s] = make_double2(zq.x / z2, -zq.y / z2);
+    }
+    if (!up(&out.col, col) || !up(&out.end, end) || !up(&out.par, par) || !up(&out.ecnt, ecnt) || !up(&out.kidx, kidx) ||
+        !up(&out.z, z) || !up(&out.y, y)) {
+        cudaGetLastError();
+        free_tree64(out);
+        return TPF_ENOMEM;
+    }
+    out.threads = th;
+    out.bpt = bpt;
+    return TPF_OK;
+}
+
 tpf_status layout_tree(tpf_handle *h, int bpt) {
     const Network &net = h->net;
     DeviceNet &d = h->dev;
     ++d.layout_gen;
     const int n = net.n_pq;
-    cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_z);
-    cudaFree(d.t_zrow); cudaFree(d.t_yrow); cudaFree(d.t_kidx); cudaFree(d.t_zrow_f); cudaFree(d.t_z64); cudaFree(d.t_y64);
+    free_tree64(d.t64);
+    free_tree64(d.t64_plain);
+    cudaFree(d.t_z); cudaFree(d.t_zrow); cudaFree(d.t_yrow); cudaFree(d.t_zrow_f);
     cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
-    d.t_z64 = d.t_y64 = nullptr;
     d.t_topo = nullptr;
     d.t_cp = nullptr;
     d.t_zf = nullptr;
-    d.t_col = d.t_end = d.t_par = d.t_ecnt = d.t_kidx = nullptr;
     d.t_z = d.t_zrow = nullptr;
     d.t_yrow = d.t_zrow_f = nullptr;
-    d.t_threads = d.t_bpt = d.t64_threads = d.t64_bpt = 0;
+    d.t_threads = d.t_bpt = 0;
     if (net.radial) {
         // Slot-ordered depth-first arrays of the sparse formulation.
         const int th = bpt ? tree_threads(n, bpt) : 0;
@@ -71,48 +124,24 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
             auto slot = [th, bpt](int q) { return (q % bpt) * th + q / bpt; };
             const int ph = net.phases, nb = n / ph;
             std::vector<int> col(ns, -1), end(ns, 0), par(ns, -1);
-            // The FP64 sparse kernel's own layout (its sums are exact, so its results do not depend on it).
-            d.t64_fixed = ph == 1 && fixed_limits(net, d.t64_z_e, d.t64_cur_max, d.t64_cur_min);
-            const int bpt64 = bpt == kTreeBigBPT ? bpt : tree64_bpt(n, d.t64_fixed), th64 = bpt64 == bpt ? th : tree_threads(n, bpt64);
-            const int ns64 = th64 * bpt64;
-            auto slot64 = [th64, bpt64](int q) { return (q % bpt64) * th64 + q / bpt64; };
-            std::vector<int> col64(ns64, -1), end64(ns64, 0), par64(ns64, -1), ecnt(ns64, 0), kidx(ns64, -1);
-            d.t64_threads = th64;
-            d.t64_bpt = bpt64;
-            int n_ends = 0;  // entries of the ends lists laid out so far, in position order
             std::vector<float4> z(ns, make_float4(0.f, 0.f, 0.f, 0.f));
-            std::vector<double2> z64(ph == 1 ? ns64 : 0, make_double2(0.0, 0.0)), y64 = z64;
             // Polyphase: row p of the branch's impedance (double-float) and admittance per slot.
             std::vector<float4> zrow(ph > 1 ? (size_t)ns * ph : 0, make_float4(0.f, 0.f, 0.f, 0.f));
             std::vector<float2> yrow(ph > 1 ? (size_t)ns * ph : 0, make_float2(0.f, 0.f)), zrow_f = yrow;
-            std::vector<int> pos_par(n, -1);  // parent position of each position
-            for (int q = 0; q < n; ++q)
-                for (int c = q + 1; c < net.dfs_end[q]; c = net.dfs_end[c]) pos_par[c] = q;
+            const std::vector<int> pos_par = parent_positions(net);
             bool fits = true;
             for (int q = 0; q < n; ++q) {
-                const int s = slot(q), cnt = net.dfs_eptr[q + 1] - net.dfs_eptr[q];
+                const int s = slot(q);
                 col[s] = net.dfs_col[q];
                 end[s] = net.dfs_end[q];
                 par[s] = pos_par[q] < 0 ? -1 : slot(pos_par[q]);
-                if (n_ends > 0xffff || cnt > 0x3fff) fits = false;
-                // start | count << 16 | phase << 30
-                const int s64 = slot64(q);
-                col64[s64] = net.dfs_col[q];
-                end64[s64] = net.dfs_end[q];
-                par64[s64] = pos_par[q] < 0 ? -1 : slot64(pos_par[q]);
-                ecnt[s64] = n_ends | (cnt << 16) | ((q / nb) << 30);
-                for (int k = net.dfs_eptr[q]; k < net.dfs_eptr[q + 1]; ++k)
-                    kidx[slot64(net.dfs_ends[k])] = n_ends++;  // where its branch term is scattered
+                if (net.dfs_eptr[q] > 0xffff || net.dfs_eptr[q + 1] - net.dfs_eptr[q] > 0x3fff) fits = false;
                 auto dd = [](double re, double im) {
                     const float rh = (float)re, ih = (float)im;
                     return make_float4(rh, ih, (float)(re - (double)rh), (float)(im - (double)ih));
                 };
                 if (ph == 1) {
                     z[s] = dd(net.dfs_z[2 * q], net.dfs_z[2 * q + 1]);
-                    const double2 zq = make_double2(net.dfs_z[2 * q], net.dfs_z[2 * q + 1]);
-                    const double z2 = zq.x * zq.x + zq.y * zq.y;
-                    z64[s64] = zq;
-                    y64[s64] = make_double2(zq.x / z2, -zq.y / z2);
                 } else {
                     for (int pp = 0; pp < ph; ++pp) {
                         const size_t k = (size_t)q * ph + pp;
@@ -154,17 +183,14 @@ tpf_status layout_tree(tpf_handle *h, int bpt) {
                 topo[s].y = cp[s];
                 zf[s] = make_float2(z[s].x, z[s].y);
             }
-            auto up = [](auto **dst, const auto &v) -> bool {
-                using T = typename std::decay_t<decltype(v)>::value_type;
-                if (cudaMalloc((void **)dst, sizeof(T) * v.size()) != cudaSuccess) return false;
-                return cudaMemcpy(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice) == cudaSuccess;
-            };
+            d.t64_fixed = ph == 1 && fixed_limits(net, d.t64_z_e, d.t64_cur_max, d.t64_cur_min);
+            // The FP64 sparse kernel has a layout of its own (its sums are exact, so its results do not depend on it).
             if (!fits) {
                 d.t_threads = 0;
-            } else if (!up(&d.t_col, col64) || !up(&d.t_end, end64) || !up(&d.t_par, par64) || !up(&d.t_ecnt, ecnt) ||
-                       !up(&d.t_z, z) || !up(&d.t_kidx, kidx) || !up(&d.t_topo, topo) || !up(&d.t_cp, cp) ||
-                       !up(&d.t_zf, zf) ||
-                       (ph == 1 && (!up(&d.t_z64, z64) || !up(&d.t_y64, y64))) || (ph > 1 && (!up(&d.t_zrow, zrow) || !up(&d.t_yrow, yrow) || !up(&d.t_zrow_f, zrow_f)))) {
+            } else if (!up(&d.t_z, z) || !up(&d.t_topo, topo) || !up(&d.t_cp, cp) || !up(&d.t_zf, zf) ||
+                       (ph == 1 && bpt != kTreeBigBPT &&
+                        layout_tree64(net, tree64_bpt(n, d.t64_fixed), d.t64) != TPF_OK) ||
+                       (ph > 1 && (!up(&d.t_zrow, zrow) || !up(&d.t_yrow, yrow) || !up(&d.t_zrow_f, zrow_f)))) {
                 cudaGetLastError();
                 d.t_threads = 0;  // no layout
                 return TPF_ECUDA;
@@ -421,8 +447,9 @@ void free_device(tpf_handle *h) {
     cudaFree(d.K64); cudaFree(d.W64); cudaFree(d.row_ptr); cudaFree(d.nbr); cudaFree(d.row_order); cudaFree(d.y64); cudaFree(d.y2f);
     cudaFree(d.Kr16); cudaFree(d.Ki16); cudaFree(d.Kd16); cudaFree(d.k_col_order);
     cudaFree(d.r_topo); cudaFree(d.r_inner); cudaFree(d.r_ypar);
-    cudaFree(d.t_col); cudaFree(d.t_end); cudaFree(d.t_par); cudaFree(d.t_ecnt); cudaFree(d.t_z);
-    cudaFree(d.t_kidx); cudaFree(d.t_z64); cudaFree(d.t_y64); cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
+    free_tree64(d.t64);
+    free_tree64(d.t64_plain);
+    cudaFree(d.t_z); cudaFree(d.t_topo); cudaFree(d.t_cp); cudaFree(d.t_zf);
     cudaFree(d.zip64); cudaFree(d.t_zip_hi); cudaFree(d.t_zip_lo);
     cudaFree(d.csr_self); cudaFree(d.vs64); cudaFree(d.t_zrow); cudaFree(d.t_yrow); cudaFree(d.t_zrow_f);
     d = DeviceNet();

@@ -839,7 +839,7 @@ tpf_status tpf_solve_batch(int F, tpf_handle *const *hs, const int64_t *T, const
         const bool sparse_ok = o.method == TPF_METHOD_SPARSE && df.radial && df.t_threads > 0 &&
                                (o.precision == TPF_PREC_MIXED ||
                                 (df.phases == 1 && df.t_bpt != tpf::kTreeBigBPT &&
-                                 tpf::tree64_smem(df.t64_threads, df.t64_bpt) <= 227 * 1024));
+                                 tpf::tree64_smem(df.t64.threads, df.t64.bpt) <= 227 * 1024));
         if (!sparse_ok) of.method = TPF_METHOD_DENSE;
         st = tpf_solve(hs[f], T[f], S_dev[f], V_dev[f], iters_dev ? iters_dev[f] : nullptr,
                        mismatch_dev ? mismatch_dev[f] : nullptr, &of, stream);

@@ -108,6 +108,14 @@ tpf_status build_network(int n_bus, int n_branch, const int32_t *from, const int
                          const int32_t *pq_bus, Network &net);
 
 // Device copies owned by a handle.
+// Slot arrays of the FP64 sparse kernel (tpf_tree64.cu), as described for DeviceNet's sparse formulation.
+struct Tree64 {
+    int threads = 0, bpt = 0;
+    int *col = nullptr, *end = nullptr, *par = nullptr, *ecnt = nullptr;
+    int *kidx = nullptr;  // per slot: the index in ends order at which its position appears, or -1
+    double2 *z = nullptr, *y = nullptr;  // z and 1 / z
+};
+
 struct DeviceNet {
     int n = 0;           // n_pq
     int n_pad = 0;       // n rounded up to kTileM (and hence to kChunkK)
@@ -132,12 +140,11 @@ struct DeviceNet {
     // subtree range ends at q, and the double-float z of the branch to the parent
     // (re_hi, im_hi, re_lo, im_lo).
     int t_threads = 0, t_bpt = 0;
-    // t_col to t_kidx, t_z64 and t_y64 are the FP64 sparse kernel's, laid out for its own block shape.
-    int t64_threads = 0, t64_bpt = 0;
+    // The FP64 sparse kernel's arrays, laid out for its own block shape, and (made when first needed) for that of
+    // the columns that leave its two-bus layout.
+    Tree64 t64, t64_plain;
     bool t64_fixed = false;  // its integers can serve, and their limits (fixed_limits, tpf_tree64.cu)
     int t64_z_e = 0, t64_cur_max = 0, t64_cur_min = 0;
-    int *t_col = nullptr, *t_end = nullptr, *t_par = nullptr, *t_ecnt = nullptr;
-    int *t_kidx = nullptr;  // per slot: the index in ends order at which its position appears, or -1
     float4 *t_z = nullptr;
     // What the mixed kernel reads of a slot when it sets a column up, as one 16-byte word: the range
     // word, column | parent slot << 16, the ends word (tpf_sparse.cu), 0; the second words again on
@@ -145,7 +152,6 @@ struct DeviceNet {
     int4 *t_topo = nullptr;
     int *t_cp = nullptr;
     float2 *t_zf = nullptr;
-    double2 *t_z64 = nullptr, *t_y64 = nullptr;  // FP64 z and 1 / z per slot (single phase), FP64 sparse kernel
     // ZIP load coefficients (Eq. 3), set by tpf_set_zip; null for constant power.  zip64: double
     // [3][n] in column order (FP64 path); t_zip_hi / t_zip_lo: float4 (alpha_P, alpha_I, alpha_Z, 0)
     // per slot, high and low words (sparse path).
@@ -333,6 +339,8 @@ tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_
                         double *mismatch, const tpf_opts &o, cudaStream_t st);
 size_t tree64_smem(int threads, int bpt);
 int tree64_bpt(int n, bool fixed);
+tpf_status layout_tree64(const Network &net, int bpt, Tree64 &out);  // single phase
+void free_tree64(Tree64 &t);
 bool fixed_limits(const Network &net, int &z_e, int &cur_max, int &cur_min);
 tpf_status solve_batch_sparse(int F, tpf_handle *const *hs, const int64_t *T, const void *const *S,
                               void *const *V, int32_t *const *iters, double *const *mismatch,

@@ -42,6 +42,7 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxWarps64 = kTreeMaxThreads / 32;
+constexpr int kCntLeft = 6;
 
 struct Tree64Args {
     int n, max_iter;
@@ -63,7 +64,9 @@ struct Tree64Args {
     int given;
     int32_t *iters_out;    // [T] or null
     double *mismatch_out;  // [T] or null
-    int *counters;         // [kCntConverged] converged columns, [5] largest sweep count
+    int *counters;         // [kCntConverged] converged columns, [5] largest sweep count, [kCntLeft]
+    const int *list;       // the columns of the launch, or null: 0, 1, ...
+    int *left;             // not null: takes the columns that leave the integers, kCntLeft of them (tree64_bpt)
 };
 
 __device__ __forceinline__ double2 dadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
@@ -184,7 +187,7 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
     longlong2 *const wti = reinterpret_cast<longlong2 *>(wt);
     __shared__ double wm[kMaxWarps64];
     __shared__ unsigned wu[kMaxWarps64];
-    const int64_t t = blockIdx.x;
+    const int64_t t = g.list ? g.list[blockIdx.x] : (int)blockIdx.x;
     const int base = tid * kBPT;
     const double2 *S = g.S + t * n;
     double2 *Vc = g.V + t * n;
@@ -255,6 +258,13 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
 
     int it = 0;
     bool conv = false;
+    auto leave = [&] {
+        if (tid == 0) g.left[atomicAdd(&g.counters[kCntLeft], 1)] = (int)t;
+    };
+    if (kBPT == 2 && !fixed && g.left) {
+        leave();
+        return;
+    }
     for (;;) {
         if (fixed) {
             longlong2 loc[kBPT], run = make_longlong2(0, 0);
@@ -337,6 +347,10 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
             mu = wu[0];
             for (int w = 1; w < nw; ++w) mu = max(mu, wu[w]);
             if (mu == ~0u) {  // every thread alike: from the start again in FP64
+                if (kBPT == 2 && g.left) {
+                    leave();
+                    return;
+                }
                 fixed = false;
                 it = 0;
 #pragma unroll
@@ -603,11 +617,13 @@ size_t tree64_smem(int threads, int bpt) {
 // Buses per thread: two up to 512 buses (256 threads), where a thread's chain of sums and products is what a
 // column waits for; four up to 2,048, eight beyond (32 B of prefix sums and loads a slot).  In us, two against
 // four: 33 buses x 16,384 columns 196 and 389, 64 buses 228 and 434, 129 x 8,000 333 and 497, 299 buses 572 and 699,
-// 512 buses 865 and 872, 699 buses 1,487 and 1,287.  In FP64 throughout a thread's scans cost more than the chain:
-// 199 buses x 4,096 columns behind a source of 12.66 (kV) take 1,615 us at two and 1,345 at four.
+// 512 buses 865 and 872, 699 buses 1,487 and 1,287.  In FP64 throughout a thread's scans cost more than the chain,
+// and two pay for the one warp of up to 64 buses only (us, two against four, behind a source of 12.66 kV): 64 buses
+// x 16,384 columns 1,221 and 1,977, 96 x 8,192 1,344 and 1,127, 256 x 8,192 3,126 and 2,557, 512 x 4,096 3,589 and
+// 2,776.  From 65 buses on a column that leaves the integers is therefore solved by a launch of its own at four.
 int tree64_bpt(int n, bool fixed) {
     for (int b : {2, 4, 8})
-        if ((b > 2 || (fixed && n <= 512)) && tree_threads(n, b)) return b;
+        if ((b > 2 || n <= (fixed ? 512 : 64)) && tree_threads(n, b)) return b;
     return 0;
 }
 
@@ -674,10 +690,9 @@ bool fixed_limits(const Network &net, int &z_e, int &cur_max, int &cur_min) {
 tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_t *iters, double *mismatch,
                         const tpf_opts &o, cudaStream_t st) {
     const DeviceNet &d = h->dev;
-    if (!d.radial || d.phases != 1 || d.t_threads == 0 || d.t_bpt == kTreeBigBPT || !d.t_z64) return TPF_EUNSUPPORTED;
+    if (!d.radial || d.phases != 1 || d.t_threads == 0 || d.t_bpt == kTreeBigBPT || !d.t64.z) return TPF_EUNSUPPORTED;
     if (T > 0x7fffffff) return TPF_EUNSUPPORTED;  // one block per column
-    const size_t smem = tree64_smem(d.t64_threads, d.t64_bpt);
-    if (smem > 227 * 1024) return TPF_EUNSUPPORTED;
+    if (tree64_smem(d.t64.threads, d.t64.bpt) > 227 * 1024) return TPF_EUNSUPPORTED;
     tpf_status rs = ensure_workspace(h, T, kWsState);  // counters
     if (rs != TPF_OK) return rs;
     Workspace &w = h->ws;
@@ -698,13 +713,6 @@ tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_
     g.cur_max = d.t64_cur_max;
     g.cur_min = d.t64_cur_min;
     if (g.fixed) g.vs_fx = make_longlong2(llrint(ldexp(g.vs.x, kFx)), llrint(ldexp(g.vs.y, kFx)));
-    g.col = d.t_col;
-    g.end = d.t_end;
-    g.par = d.t_par;
-    g.ecnt = d.t_ecnt;
-    g.kidx = d.t_kidx;
-    g.z = d.t_z64;
-    g.y = d.t_y64;
     g.zip = d.zip64;
     g.S = static_cast<const double2 *>(S);
     g.V = static_cast<double2 *>(V);
@@ -713,27 +721,61 @@ tpf_status solve_tree64(tpf_handle *h, int64_t T, const void *S, void *V, int32_
     g.mismatch_out = mismatch;
     g.counters = w.counters;
     KernelTimer timer(o.profile != 0, st);
-    timer.begin(KernelTimer::kGemm);
-    cudaError_t e;
-    switch (d.t64_bpt) {
-        case 2: e = launch64<2>(d.t64_threads, T, smem, g, st); break;
-        case 4: e = launch64<4>(d.t64_threads, T, smem, g, st); break;
-        case 8: e = launch64<8>(d.t64_threads, T, smem, g, st); break;
-        default: return TPF_EUNSUPPORTED;
+    auto run = [&](const Tree64 &l, int64_t cols) {
+        g.col = l.col;
+        g.end = l.end;
+        g.par = l.par;
+        g.ecnt = l.ecnt;
+        g.kidx = l.kidx;
+        g.z = l.z;
+        g.y = l.y;
+        const size_t smem = tree64_smem(l.threads, l.bpt);
+        timer.begin(KernelTimer::kGemm);
+        cudaError_t e;
+        switch (l.bpt) {
+            case 2: e = launch64<2>(l.threads, cols, smem, g, st); break;
+            case 4: e = launch64<4>(l.threads, cols, smem, g, st); break;
+            case 8: e = launch64<8>(l.threads, cols, smem, g, st); break;
+            default: return TPF_EUNSUPPORTED;
+        }
+        timer.end();
+        if (e != cudaSuccess || cudaGetLastError() != cudaSuccess ||
+            cudaMemcpyAsync(w.counters_host, w.counters, sizeof(int) * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess) {
+            cudaGetLastError();
+            return TPF_ECUDA;
+        }
+        return TPF_OK;
+    };
+    const bool leaves = d.t64.bpt < tree64_bpt(d.n, false);
+    g.left = leaves ? w.flags : nullptr;
+    auto plain = [&]() -> tpf_status {  // the layout of the columns that leave
+        if (d.t64_plain.z) return TPF_OK;
+        try {
+            return layout_tree64(h->net, tree64_bpt(d.n, false), h->dev.t64_plain);
+        } catch (const std::bad_alloc &) {
+            return TPF_ENOMEM;
+        }
+    };
+    int launches = 1;
+    if (leaves && !g.fixed) {
+        rs = plain();
+        if (rs == TPF_OK) rs = run(d.t64_plain, T);
+    } else {
+        rs = run(d.t64, T);
+        if (rs == TPF_OK && w.counters_host[kCntLeft] > 0) {
+            rs = plain();
+            g.list = w.flags;
+            g.left = nullptr;
+            g.fixed = 0;
+            if (rs == TPF_OK) rs = run(d.t64_plain, w.counters_host[kCntLeft]);
+            ++launches;
+        }
     }
-    timer.end();
-    if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) {
-        cudaGetLastError();
-        return TPF_ECUDA;
-    }
-    if (cudaMemcpyAsync(w.counters_host, w.counters, sizeof(int) * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
-        cudaGetLastError();
-        return TPF_ECUDA;
-    }
+    if (rs != TPF_OK) return rs;
     const int64_t conv = w.counters_host[kCntConverged];
     h->stats.sweeps = w.counters_host[5];
-    h->stats.kernel_launches = 1;
+    h->stats.kernel_launches = launches;
     h->stats.converged = conv;
     h->stats.gemm_ms = timer.total_ms(KernelTimer::kGemm);
     return conv == T ? TPF_OK : TPF_ENOCONV;
