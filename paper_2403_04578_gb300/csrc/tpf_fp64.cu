@@ -413,7 +413,8 @@ tpf_status set_zip(tpf_handle *h, const double *alpha) {
     if (d.phases > 1) return alpha ? TPF_EUNSUPPORTED : TPF_OK;
     ++d.layout_gen;
     // The sparse kernel's ZIP coefficients take a fourth shared-memory region (16 B per slot): at 8
-    // buses per thread (3,073 to 4,096 demand buses) the block would need more than 227 KB, so such
+    // buses per thread the block needs more than 227 KB from 3,329 demand buses on, and the rule, which
+    // counts 2 B a slot more than the kernel takes, moves those from 3,073 on: such
     // feeders are laid out at 16 buses per thread, whose kernel keeps the coefficients in device
     // scratch; without coefficients they return to the default layout.
     if (d.radial && d.t_threads > 0) {

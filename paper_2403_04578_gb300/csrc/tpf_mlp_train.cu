@@ -117,25 +117,23 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_gemm(const __grid_constant__ 
     const uint32_t tmem = *tmem_slot;
     volatile int *vabort = abort_flag;
 
-    constexpr int c0 = 0;
-    int p = 0, m0, n0, c1;
+    const int chunks = g.chunks;
+    int p = 0, m0, n0;
     if constexpr (KIND == kWgrad) {
         while (p + 1 < g.layers && (int)blockIdx.x >= g.first[p + 1]) ++p;
         const int tile = (int)blockIdx.x - g.first[p];
         m0 = (tile % g.m_tiles[p]) * kTileM;
         n0 = (tile / g.m_tiles[p]) * kN;
-        c1 = g.chunks;
     } else {
         m0 = (int)blockIdx.y * kTileM;
         n0 = (int)blockIdx.x * kN;
-        c1 = g.chunks;
     }
 
     if (warp == 0) {
         if (lane == 0) {
             const uint32_t sbase = smem_u32(smem);
             int k = 0;
-            for (int c = c0; c < c1; ++c, ++k) {
+            for (; k < chunks; ++k) {
                 const int slot = k % R::kStages;
                 if (!mbar_wait(smem_u32(&empty[slot]), ((uint32_t)(k / R::kStages) & 1) ^ 1)) {
                     *vabort = 1;
@@ -144,8 +142,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_gemm(const __grid_constant__ 
                 }
                 const uint32_t st = sbase + slot * R::kStage, bar = smem_u32(&full[slot]);
                 mbar_expect_tx(bar, R::kStage);
-                tma_load_2d(st, map_a(g, p), bar, c * kChunkK, m0);
-                tma_load_2d(st + kABytes, map_b(g, p), bar, c * kChunkK, n0);
+                tma_load_2d(st, map_a(g, p), bar, k * kChunkK, m0);
+                tma_load_2d(st + kABytes, map_b(g, p), bar, k * kChunkK, n0);
             }
             if (*vabort)
                 for (int q = k - 1; q >= 0 && q >= k - R::kStages; --q)
@@ -155,7 +153,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_gemm(const __grid_constant__ 
         const uint32_t sbase = smem_u32(smem), id = idesc_f16(kTileM, kN, 0, 1);
         const bool lead = elect_one();
         uint32_t slot = 0, phase = 0;
-        for (int c = c0; c < c1; ++c) {
+        for (int c = 0; c < chunks; ++c) {
             if (!mbar_wait(smem_u32(&full[slot]), phase)) {
                 if (lead) {
                     *vabort = 1;
@@ -168,7 +166,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_gemm(const __grid_constant__ 
             if (lead) {
 #pragma unroll
                 for (int kk = 0; kk < kChunkK / 16; ++kk)
-                    umma_f16(tmem, da + kk * 2, da + kABytes / 16 + kk * 2, id, c != c0 || kk != 0);
+                    umma_f16(tmem, da + kk * 2, da + kABytes / 16 + kk * 2, id, c != 0 || kk != 0);
                 umma_commit(smem_u32(&empty[slot]));
             }
             __syncwarp();
@@ -469,7 +467,6 @@ tpf_status launch_adam(AdamArgs &g, cudaStream_t st) {
         g.l[i].tile0 = tiles;
         tiles += g.l[i].Po / 32 * (g.l[i].Pi / 32);
     }
-    g.tiles = tiles;
     return launch_pdl(mlp_adam, dim3((unsigned)tiles), kAdamThreads, 0, st, g);
 }
 

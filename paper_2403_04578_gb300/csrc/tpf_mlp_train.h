@@ -53,7 +53,7 @@ struct AdamLayer {
 };
 struct AdamArgs {
     AdamLayer l[kTrainLayers];
-    int L, tiles, update;
+    int L, update;
     float lr, b1, b2, eps, c1, c2;
 };
 tpf_status launch_adam(AdamArgs &g, cudaStream_t st);

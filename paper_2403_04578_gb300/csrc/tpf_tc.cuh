@@ -1,7 +1,7 @@
 // Inline-PTX wrappers for the tcgen05 kernels (sm_103a): shared-memory mbarriers with bounded
 // waits, TMA tile loads, UMMA shared-memory and instruction descriptors, tcgen05.mma issue and
-// commit, and tcgen05.ld of accumulator lanes.  Used by the complex GEMM of the mixed path and
-// the fused inference kernel of the learned start.
+// commit, and tcgen05.ld of accumulator lanes.  Used by the complex GEMM of the mixed path, the
+// fixed-point product of the FP64 path and the learned start's training and inference kernels.
 #pragma once
 
 #include <cuda.h>

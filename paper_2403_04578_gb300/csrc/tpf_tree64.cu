@@ -13,9 +13,11 @@
 // (max_i |V_{k+1,i} - V_{k,i}| <= tol, the first iterate that meets it is returned), so that it can stand
 // beside the mixed-precision sparse path as a like-for-like FP64 reference.
 //
-// GB300 issues FP64 at 1/64 of its FP32 rate, and the FP64 pipe is what bounds this kernel.  Only the
-// products and the division need it: every sum runs in 64-bit fixed point, two integer instructions
-// instead of an FP64 one that takes sixteen times as long.  Currents are integers of a last place
+// GB300 issues FP64 at 1/64 of its FP32 rate, and with every operation on that pipe it bounds this kernel
+// (16,384 columns of 1,000 buses in 16.6 ms).  So the sums run in 64-bit fixed point, two integer
+// instructions instead of an FP64 one that takes sixteen times as long, the load currents are integer
+// quotients (tpf_fx.cuh) and the branch terms 128-bit integer products: 3.5 ms, bound by issue slots.  ZIP
+// currents and the balance at the end stay in FP64.  Currents are integers of a last place
 // 2^cur that the sum over all buses cannot overflow (per column, from its largest load), branch terms,
 // path sums and V integers of 2^-61 pu.  Integer sums are exact, so what an FP64 prefix sum loses at its
 // own magnitude is not lost; V is rounded to FP64 where it enters a product and where it is returned.
@@ -193,8 +195,6 @@ __global__ void __launch_bounds__(kTreeMaxThreads) __maxnreg__(kBPT == 4 ? 80 : 
     double2 *Vc = g.V + t * n;
 
     double2 V[kBPT];  // in fixed point the bits of two integers of 2^-61 pu
-#pragma unroll
-    for (int j = 0; j < kBPT; ++j) V[j] = make_double2(1.0, 0.0);  // flat start (Algorithm 1)
     int ecnt[kBPT];
     unsigned smax = 0;  // largest high word of the thread's loads
     auto get_v = [&V](int j) { return make_longlong2(__double_as_longlong(V[j].x), __double_as_longlong(V[j].y)); };
