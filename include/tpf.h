@@ -54,7 +54,8 @@ typedef enum {
 enum {
     TPF_PREC_FP64 = 0,  /* the plain fixed-point iteration (direct form) with every iterate to     *
                          * double-precision rounding; its sums and the dense product run in exact *
-                         * fixed point where that is faster than the FP64 units                   */
+                         * fixed point where that is faster than the FP64 units and at least as   *
+                         * fine, column by column                                                 */
     TPF_PREC_MIXED = 1  /* fp16 tensor-core sweeps with FP32 accumulation in residual form         *
                          * V <- V + K rho(V); V is carried as two floats and rho is evaluated    *
                          * against a double-float anchor, so results reach FP64-level accuracy  */

@@ -171,7 +171,7 @@ __device__ __forceinline__ float scaled_f(double v, int u) {
 // power of two, so J is the current of a load c_j S.
 // Constant-power currents of voltages from 0.5 to 2 pu come from integer remainders (current_fx), the others, ZIP loads
 // and columns out of its range from FP64 divisions, which bound the kernel: 23.7 instead of 30.2 us for 4,800
-// columns of 199 buses (the bytes of S, V and the planes take 13), 1.83 instead of 1.92 ms for a solve of 8,760.
+// columns of 199 buses (the bytes of S, V and the planes take 13), 27.3 with the scales c_j; integer pipe 68 % active.
 __global__ void __launch_bounds__(kSliceThreads)
     fx_slice(int n, int n_pad, const int *__restrict__ list, const int *count, int first,
              const double2 *__restrict__ S,

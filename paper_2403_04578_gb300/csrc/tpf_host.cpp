@@ -448,7 +448,7 @@ tpf_status host_chunks(tpf_handle *h, int64_t T, const void *S_host, void *V_hos
     // at once on an input stream, each chunk's solve waits only for its own copy, and its results go
     // back on an output stream while the next chunk is solved (pinned host memory overlaps; pageable
     // memory still works, with the copies serialised by the driver).
-    // The copies cost about three times the sparse solve, so its chunks only have to be large enough for their
+    // The copies cost about three times the mixed sparse solve (and slower kernels only weigh more), so its chunks only have to be large enough for their
     // fill, drain and host round trip (100 us) not to count: sqrt(3 MB times all bytes), 16 MB at least and 32
     // chunks at most.  Pinned, 20,160 columns of 999 buses (322 MB each way) take 4.86 ms in one chunk, 2.66 in
     // chunks of 32 MB, 2.90 of 16 and 3.75 of 8; 5,000 columns 1.29 ms, 0.88 of 24, 0.90 of 16; 86,400 of 99
