@@ -17,7 +17,7 @@
 // (16,384 columns of 1,000 buses in 16.6 ms).  So the sums run in 64-bit fixed point, two integer
 // instructions instead of an FP64 one that takes sixteen times as long, the load currents are integer
 // quotients (tpf_fx.cuh) and the branch terms 128-bit integer products: 3.5 ms, bound by issue slots.  ZIP
-// currents and the balance at the end stay in FP64.  Currents are integers of a last place
+// currents and the products of the balance at the end stay in FP64.  Currents are integers of a last place
 // 2^cur that the sum over all buses cannot overflow (per column, from its largest load), branch terms,
 // path sums and V integers of 2^-61 pu.  Integer sums are exact, so what an FP64 prefix sum loses at its
 // own magnitude is not lost; V is rounded to FP64 where it enters a product and where it is returned.
@@ -634,9 +634,10 @@ int tree64_bpt(int n, bool fixed) {
 // mean square; the sums of squares grow along a path.  The feeders of inputs.py are 21 times below that (1,000
 // buses).  One load of thousands of times the others is not: such columns lost 3.3e-14 pu (1,000 pu beside 399
 // ordinary loads) to 3.0e-11 (1e6 pu).
-// Impedances above 2^8 times the median set neither z_e nor the limit, but a column with a current there goes to
-// FP64 (the kernel looks).  Most are open switches, without a current: a stub of 1e6 pu cost the others 7.4e-13 pu
-// when it set the place of all impedances, one of 1e12 pu 7.9e-7.
+// Impedances above 2^8 times the upper quartile set neither z_e nor the limit, but a column with a current there goes
+// to FP64 (the kernel looks).  Most are open switches, without a current: a stub of 1e6 pu cost the others 7.4e-13 pu
+// when it set the place of all impedances, one of 1e12 pu 7.9e-7.  (Not the median: more than half of a feeder's
+// branches may be couplers of next to no impedance, and its lines must not count as large.)
 // cur_min is for the mismatch alone: a bus's branch currents are off by up to 2^-50 sum |y| (V is returned to 2^-52
 // pu), and 2^61 integers hold that beside the currents.  Only branches of 1e-14 pu and less, or loads as small,
 // come near (the sums wrapped there, and the mismatch was reported as 16 instead of 29).
@@ -646,8 +647,8 @@ bool fixed_limits(const Network &net, int &z_e, int &cur_max, int &cur_min) {
     std::vector<int> e(n);
     for (int q = 0; q < n; ++q) frexp(std::max(std::fabs(net.dfs_z[2 * q]), std::fabs(net.dfs_z[2 * q + 1])), &e[q]);
     std::vector<int> by_size = e;
-    std::nth_element(by_size.begin(), by_size.begin() + n / 2, by_size.end());
-    const int cut = by_size[n / 2] + 8;
+    std::nth_element(by_size.begin(), by_size.begin() + 3 * n / 4, by_size.end());
+    const int cut = by_size[3 * n / 4] + 8;
     z_e = -2000;
     for (int v : e)
         if (v <= cut) z_e = std::max(z_e, v);
